@@ -358,6 +358,17 @@ std::vector<int> tile_candidates(int model, int narr, int esz, int N, size_t sme
   return out;
 }
 
+// What a plane of a tile costs its CTA (choose_tiles in worklist.h), from passes of
+// 1 to 8 planes per CTA at 32^3 to 96^3: FP32 planes are bound by latency (1.1 us at
+// 512 sites, 1.25 us at 2048), U(1) planes take 2.0 us at 512 sites and 3.0 us at
+// 1024, FP64 planes go by the FP64 pipe (one field 2.0 us at 256 sites, 5.8 us at
+// 1024; two fields 5.7 us at 512, 10.5 us at 1024).
+PlaneCost plane_cost(const cl_ctx* c) {
+  const int fields = c->model == CL_MODEL_U1_HIGGS ? 16 : c->nf;  // FP64: U(1)'s sines cost several times its products
+  if (!c->fp32) return PlaneCost{1.2, 0.0045 * fields};
+  return c->model == CL_MODEL_U1_HIGGS ? PlaneCost{1.0, 0.002} : PlaneCost{1.0, 0.0001 * fields};
+}
+
 // Device copy of pass weights, cached by content.
 cl_status device_steps(cl_ctx* c, const PassStep* st, int n, const PassStep** out) {
   std::vector<PassStep> key(st, st + n);
@@ -848,6 +859,7 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
   // least 3 stages of BY + 2 rows of every array in shared memory
   c->lats.resize(c->nlat);
   std::vector<LatTiles> tiles;
+  std::vector<std::vector<int>> heights;  // per lattice, the tile heights to choose from
   size_t stage = 0;
   for (int l = 0; l < c->nlat; ++l) {
     LatHost& L = c->lats[l];
@@ -866,15 +878,14 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
     } else if (c->p.autotune) {
       cl_status s = tune_tile(c, L.N, L.kIR, &L.BY);
       if (s != CL_OK) return s;
-    } else {
-      L.BY = cand[0];
     }
     tiles.push_back(LatTiles{L.N, L.BY, THREADS * tile_vx(c->model, c->esz)});
+    // a given or tuned height is the only one
+    heights.push_back(L.BY > 0 ? std::vector<int>{L.BY} : cand);
   }
-  // work list: one CTA per SM, at least 8 plane tasks each
-  long long tasks = 0;
-  for (const LatTiles& t : tiles) tasks += (long long)(t.N / t.BY) * t.N;
-  c->grid = (int)std::max<long long>(1, std::min<long long>(c->nsm, tasks / 8));
+  // work list: tile heights (where not given or tuned) and CTAs, at most one per SM
+  c->grid = choose_tiles(tiles, heights, c->nsm, u1, plane_cost(c));
+  for (int l = 0; l < c->nlat; ++l) c->lats[l].BY = tiles[l].BY;
   std::vector<Seg> segs;
   std::vector<int> cta, sbeg, send;
   if (!build_worklist(tiles, c->grid, u1, segs, cta, sbeg, send)) {
@@ -2022,12 +2033,14 @@ static cl_status adjoint_plan(cl_ctx* c) {
   const int narr = 4 * c->nf;
   const std::vector<int> cand = tile_candidates(c->model, narr, c->esz, H.N, c->smem_optin);
   if (cand.empty()) return fail(c, CL_EUNSUPPORTED, "no adjoint tile shape for N=%d", H.N);
-  const int BY = cand[0];
-  const long long tasks = (long long)(H.N / BY) * H.N;
-  A.grid = (int)std::max<long long>(1, std::min<long long>(c->nsm, tasks / 8));
+  std::vector<LatTiles> tiles = {LatTiles{H.N, 0, THREADS * tile_vx(c->model, c->esz)}};
+  PlaneCost cost = plane_cost(c);
+  cost.c1 *= 2.0;  // the state and its adjoint
+  A.grid = choose_tiles(tiles, {cand}, c->nsm, false, cost);
+  const int BY = tiles[0].BY;
   std::vector<Seg> segs;
   std::vector<int> cta, sbeg, send;
-  if (!build_worklist({LatTiles{H.N, BY, THREADS * tile_vx(c->model, c->esz)}}, A.grid, false, segs, cta, sbeg, send))
+  if (!build_worklist(tiles, A.grid, false, segs, cta, sbeg, send))
     return fail(c, CL_EUNSUPPORTED, "adjoint work split too fine");
   A.stage_bytes = (unsigned)stage_size(H.N, BY, narr, c->esz);
   A.stages = (int)std::min<size_t>(6, (c->smem_optin - SM_TAIL_BYTES) / A.stage_bytes);

@@ -237,4 +237,75 @@ inline bool build_worklist(const std::vector<LatTiles>& lats, int grid, bool up_
   return true;
 }
 
+// Tile heights and the number of CTAs of a pass.  With many planes per CTA (large
+// lattices) the tallest tiles and every SM are best.  A small lattice's pass is a
+// chain of latencies: a plane of a tile costs its CTA about c0 + c1 sites
+// microseconds however few CTAs run, so the planes are spread over as many SMs
+// as there are, in equal runs (an uneven split runs as long as its longest CTA:
+// 96^3 FP32 16.3 us per pass in 144 runs of 4 planes, 17.6 us on 152 CTAs), and a
+// tile is cut lower where that saves more than the extra planes cost (FP64, whose
+// planes cost by the site).  kFewPlanes: at 16 planes per CTA and above the two
+// agree within a few per cent and the tallest tiles on all SMs stay.  Measured
+// (us per pass, before: 8 planes or more per CTA): 32^3 FP64 58.6 -> 13.2,
+// 64^3 FP64 96.9 -> 33.7, 64^3 FP32 22.8 -> 12.5, 96^3 FP32 21.2 -> 16.3,
+// U(1) 64^3 FP32 39.2 -> 22.0.
+struct PlaneCost {
+  double c0, c1;  // microseconds per plane, and per site of the plane
+};
+constexpr double kHaloPlanes = 0.3;  // a run's two halo planes (loaded, not kicked) in planes
+constexpr int kFewPlanes = 16;
+
+// cand[l]: the admissible tile heights of lattice l, tallest first (at least one);
+// lats[l].N and .min_sites are given, .BY is chosen.  Returns the CTA count.
+inline int choose_tiles(std::vector<LatTiles>& lats, const std::vector<std::vector<int>>& cand, int nsm,
+                        bool up_only, const PlaneCost& cost) {
+  auto tasks_at = [&](int cut, std::vector<int>* by, int* sites) {
+    long long t = 0;
+    *sites = 0;
+    for (size_t l = 0; l < lats.size(); ++l) {
+      // the tallest height at most the cut-th part of the tallest
+      int b = cand[l].back();
+      for (int h : cand[l])
+        if (h * cut <= cand[l][0]) {
+          b = h;
+          break;
+        }
+      by->push_back(b);
+      t += (long long)(lats[l].N / b) * lats[l].N;
+      *sites = std::max(*sites, b * lats[l].N);
+    }
+    return t;
+  };
+  // planes of the longest run of a split, with its segments' set-up
+  auto longest = [&](int grid) {
+    std::vector<Seg> segs;
+    std::vector<int> first, sb, se;
+    if (!build_worklist(lats, grid, up_only, segs, first, sb, se)) return 1e300;
+    double worst = 0.0;
+    for (int k = 0; k < grid; ++k) {
+      double w = 0.0;
+      for (int i = first[k]; i < first[k + 1]; ++i) w += segs[i].nz + kSegCost;
+      worst = std::max(worst, w);
+    }
+    return worst;
+  };
+  double best = 0.0;
+  int grid = 1;
+  for (int cut = 1; cut <= 64; ++cut) {
+    std::vector<int> by;
+    int sites = 0;
+    const long long t = tasks_at(cut, &by, &sites);
+    const long long p = (t + nsm - 1) / nsm;
+    const double c = ((double)p + kHaloPlanes) * (cost.c0 + cost.c1 * sites);
+    if (cut > 1 && c >= best - 1e-9) continue;
+    best = c;
+    for (size_t l = 0; l < lats.size(); ++l) lats[l].BY = by[l];
+    grid = (int)(p >= kFewPlanes ? nsm : std::max<long long>(1, (t + p - 1) / p));
+    if (cut == 1 && p >= kFewPlanes) break;
+  }
+  // equal runs, unless every SM shortens the longest one
+  if (grid < nsm && longest(nsm) < longest(grid) - 1e-9) grid = nsm;
+  return grid;
+}
+
 }  // namespace clg
