@@ -108,7 +108,7 @@ struct LatHost {
 // the reversed-pass kernel's own tiling over the state and adjoint arrays.
 struct AdjPlan {
   bool ready = false;
-  int grid = 0, stages = 0;
+  int grid = 0, stages = 0, nseg_max = 0, nrun_max = 0;
   unsigned stage_bytes = 0;
   size_t smem = 0;
   bool coop = false;
@@ -167,7 +167,7 @@ struct cl_ctx {
   std::vector<std::pair<std::vector<PassStep>, void*>> step_cache;
   std::vector<GraphEntry> graph_cache;
   AdjPlan adj;
-  int grid = 0, nseg = 0, nslot = 0, stages = 0;
+  int grid = 0, nseg = 0, nseg_max = 0, nrun_max = 0, nslot = 0, stages = 0;
   unsigned stage_bytes = 0;
   size_t smem_bytes = 0;
   int su2_kd_ty = 8;                // doublet models: tile height of the kick-then-drift step pass (RED 0)
@@ -344,6 +344,10 @@ size_t stage_size(int N, int BY, int narr, int esz, bool mown = false) {
 // the own sites only, so their stages hold the momenta without halo rows.
 bool ring_mown(const cl_ctx* c) { return c->model == CL_MODEL_U1_HIGGS && c->p.expansion != CL_EXP_SELF; }
 
+// Shared memory that tile_candidates sets aside behind the stages: what a CTA of
+// MAX_SEG_PER_CTA segments over a few dozen lattices needs.
+constexpr size_t SM_TAIL_RESERVE = 17408;
+
 // Tile heights BY admissible for N: BY divides N, the BY rows of N/VX
 // threads fit in one CTA, and at least 3 stages fit in shared memory; the
 // tallest first.
@@ -353,7 +357,7 @@ std::vector<int> tile_candidates(int model, int narr, int esz, int N, size_t sme
   if (TX > THREADS) return out;
   for (int by = std::min(N, THREADS / TX); by >= 1; --by) {
     if (N % by) continue;
-    if ((smem_optin - SM_TAIL_BYTES) / stage_size(N, by, narr, esz, mown) >= 3) out.push_back(by);
+    if ((smem_optin - SM_TAIL_RESERVE) / stage_size(N, by, narr, esz, mown) >= 3) out.push_back(by);
   }
   return out;
 }
@@ -367,6 +371,37 @@ PlaneCost plane_cost(const cl_ctx* c) {
   const int fields = c->model == CL_MODEL_U1_HIGGS ? 16 : c->nf;  // FP64: U(1)'s sines cost several times its products
   if (!c->fp32) return PlaneCost{1.2, 0.0045 * fields};
   return c->model == CL_MODEL_U1_HIGGS ? PlaneCost{1.0, 0.002} : PlaneCost{1.0, 0.0001 * fields};
+}
+
+// Lets kernel k take all the dynamic shared memory a block may have: the attribute is
+// the function's, not the context's, and contexts of other sizes share the kernel.
+cudaError_t allow_dynamic_smem(const cl_ctx* c, PassKernel k) {
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, (const void*)k);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(c->smem_optin - fa.sharedSizeBytes));
+}
+
+// Bytes of a CTA's record of one lattice: LatRun with the model's coefficients, and
+// the adjoint pass's (AdjUpdate::Rec); both are 16-byte aligned.
+size_t run_record_bytes(int model, int esz) {
+  const size_t cf = (model == CL_MODEL_U1_HIGGS ? 9 : 4) * (size_t)esz;
+  return (sizeof(ScalarState) + sizeof(LatPar) + cf + 15) / 16 * 16;
+}
+size_t adj_record_bytes(int esz) {
+  return ((5 + 2 * ADJ_COEF_W) * sizeof(double) + 8 * (size_t)esz + 15) / 16 * 16;
+}
+
+// The most segments, and the most lattices, of any CTA of a split.
+void run_counts(const std::vector<Seg>& segs, const std::vector<int>& cta, int& nseg, int& nrun) {
+  nseg = nrun = 1;
+  for (size_t k = 0; k + 1 < cta.size(); ++k) {
+    int r = 0;
+    for (int i = cta[k]; i < cta[k + 1]; ++i) r += i == cta[k] || segs[i].lat != segs[i - 1].lat;
+    nseg = std::max(nseg, cta[k + 1] - cta[k]);
+    nrun = std::max(nrun, r);
+  }
 }
 
 // Device copy of pass weights, cached by content.
@@ -482,6 +517,8 @@ cl_status launch_passes(cl_ctx* c, const PassStep* st, int n, int red, int write
   A.cta_seg = c->d_cta;
   A.partials = c->d_part;
   A.nslot = c->nslot;
+  A.nseg_max = c->nseg_max;
+  A.nrun_max = c->nrun_max;
   A.counters = c->d_cnt;
   A.ck = st[0].ck;
   A.wout = st[0].wout;
@@ -901,21 +938,40 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
     if (!ok)
       return fail(c, CL_EUNSUPPORTED, "work split needs more than %d segments per CTA", MAX_SEG_PER_CTA);
   }
+  // stage ring: the largest lattice stage, as many stages (3 .. 6) as fit beside the
+  // CTAs' records; where a CTA's records of very many lattices leave fewer than three,
+  // the lattices of the largest stage take the next lower tile
+  size_t tail = 0;
+  int S = 0;
+  for (;;) {
+    stage = 0;
+    for (const LatHost& L : c->lats) stage = std::max(stage, stage_size(L.N, L.BY, c->narr, c->esz, ring_mown(c)));
+    run_counts(segs, cta, c->nseg_max, c->nrun_max);
+    tail = sm_tail_bytes(c->nseg_max, c->nrun_max, run_record_bytes(c->model, c->esz));
+    S = (int)std::min<size_t>(6, (c->smem_optin - tail) / stage);
+    if (S >= 3) break;
+    bool lower = false;
+    for (int l = 0; l < c->nlat; ++l) {
+      LatHost& L = c->lats[l];
+      if (stage_size(L.N, L.BY, c->narr, c->esz, ring_mown(c)) != stage || L.BY == 1) continue;
+      do --L.BY;
+      while (L.N % L.BY);
+      tiles[l].BY = L.BY;
+      lower = true;
+    }
+    if (!lower || !build_worklist(tiles, c->grid, u1, segs, cta, sbeg, send))
+      return fail(c, CL_EUNSUPPORTED, "shared memory too small for the stage ring");
+  }
   c->nseg = (int)segs.size();
   c->nslot = send[c->nlat - 1];
-  // stage ring: the largest lattice stage, as many stages (3 .. 6) as fit
-  for (const LatHost& L : c->lats) stage = std::max(stage, stage_size(L.N, L.BY, c->narr, c->esz, ring_mown(c)));
-  const int S = (int)std::min<size_t>(6, (c->smem_optin - SM_TAIL_BYTES) / stage);
-  if (S < 3) return fail(c, CL_EUNSUPPORTED, "shared memory too small for the stage ring");
   c->stages = S;
   c->stage_bytes = (unsigned)stage;
-  c->smem_bytes = (size_t)S * stage + SM_TAIL_BYTES;
+  c->smem_bytes = (size_t)S * stage + tail;
   for (int red = 0; red < 3; ++red) {
     PassKernel k = pick_kernel(c, red);
     if (!k && red == 1 && red_for_step(c) == 0) continue;  // Friedmann sums never taken here
     if (!k) return fail(c, CL_EUNSUPPORTED, "no pass kernel for this configuration");
-    CU(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)c->smem_bytes));
+    CU(allow_dynamic_smem(c, k));
   }
   // device memory
   for (int l = 0; l < c->nlat; ++l) {
@@ -929,7 +985,7 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
   CU(cudaMemsetAsync(c->d_sc, 0, c->nlat * sizeof(LatScalars), c->stream));
   CU(cudaMalloc(&c->d_segs, segs.size() * sizeof(Seg)));
   CU(cudaMalloc(&c->d_cta, cta.size() * sizeof(int)));
-  CU(cudaMalloc(&c->d_part, (size_t)c->nslot * NQ * sizeof(double)));
+  CU(cudaMalloc(&c->d_part, 2 * (size_t)c->nslot * NQ * sizeof(double)));  // two sets, by the pass's parity
   CU(cudaMalloc(&c->d_cnt, c->nlat * sizeof(unsigned)));
   CU(cudaMemsetAsync(c->d_cnt, 0, c->nlat * sizeof(unsigned), c->stream));
   CU(cudaMalloc(&c->d_gsync, 2 * sizeof(unsigned)));
@@ -2043,16 +2099,19 @@ static cl_status adjoint_plan(cl_ctx* c) {
   if (!build_worklist(tiles, A.grid, false, segs, cta, sbeg, send))
     return fail(c, CL_EUNSUPPORTED, "adjoint work split too fine");
   A.stage_bytes = (unsigned)stage_size(H.N, BY, narr, c->esz);
-  A.stages = (int)std::min<size_t>(6, (c->smem_optin - SM_TAIL_BYTES) / A.stage_bytes);
-  A.smem = (size_t)A.stages * A.stage_bytes + SM_TAIL_BYTES;
+  run_counts(segs, cta, A.nseg_max, A.nrun_max);
+  const size_t tail = sm_tail_bytes(A.nseg_max, A.nrun_max, adj_record_bytes(c->esz));
+  A.stages = (int)std::min<size_t>(6, (c->smem_optin - tail) / A.stage_bytes);
+  if (A.stages < 3) return fail(c, CL_EUNSUPPORTED, "shared memory too small for the adjoint's stage ring");
+  A.smem = (size_t)A.stages * A.stage_bytes + tail;
   PassKernel k = adjoint_pass_kernel(c->fp32, c->nf, c->p.expansion == CL_EXP_SELF);
-  CU(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A.smem));
+  CU(allow_dynamic_smem(c, k));
   const size_t ab = (size_t)H.V * c->esz;
   CU(cudaMalloc(&A.lam, 2 * (size_t)(2 * c->nf) * ab));
   CU(cudaMalloc(&A.d_lat, sizeof(LatConst)));
   CU(cudaMalloc(&A.d_segs, segs.size() * sizeof(Seg)));
   CU(cudaMalloc(&A.d_cta, cta.size() * sizeof(int)));
-  CU(cudaMalloc(&A.d_part, (size_t)send[0] * NQ * sizeof(double)));
+  CU(cudaMalloc(&A.d_part, 2 * (size_t)send[0] * NQ * sizeof(double)));
   A.nslot = send[0];
   CU(cudaMalloc(&A.d_cnt, sizeof(unsigned)));
   CU(cudaMalloc(&A.d_out, 2 * sizeof(double) + 2 * c->nsm * sizeof(double)));
@@ -2093,6 +2152,8 @@ static cl_status launch_adjoint(cl_ctx* c, const double* dev_coef, int n) {
   A.cta_seg = J.d_cta;
   A.partials = J.d_part;
   A.nslot = J.nslot;
+  A.nseg_max = J.nseg_max;
+  A.nrun_max = J.nrun_max;
   A.counters = J.d_cnt;
   A.parity = c->parity;
   A.write = 1;

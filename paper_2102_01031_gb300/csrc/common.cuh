@@ -18,7 +18,7 @@ constexpr int THREADS = 32 * CONSUMER_WARPS;
 static_assert(CONSUMER_WARPS >= NQ, "the tail sums one slot per warp");
 
 // Per-lattice constants, read-only during a pass.
-struct LatConst {
+struct LatPar {
   int N, BY, YT, model, nf, narr, expansion, esz;
   int slot_begin, slot_end;  // partial-sum slots of this lattice: [slot_begin, slot_end)
   int int_alpha, alpha_i;    // int_alpha: alpha is the integer alpha_i in [-4, 4] (powers by multiplication)
@@ -29,6 +29,8 @@ struct LatConst {
   double gQB;                  // doublet model: SU(2) coupling times charge
   double qG, qH, Qc;           // lphi4SU2U1: potential couplings, charge of vphi (units of the doublet's)
   int su2_nzc, su2_pad;        // doublet model: z-chunks of the pass's work items
+};
+struct LatConst : LatPar {
   void* buf[2][MAX_ARR];  // ping-pong storage; array 2f = field f, 2f+1 = its momentum
 };
 
@@ -100,10 +102,14 @@ __device__ __forceinline__ void prefetch_l1(const T* p) {
 // Sites per thread along x in the U(1) pass (8-byte vectors in FP32, scalars in FP64).
 constexpr int u1_vx(int esz) { return esz == 4 ? 2 : 1; }
 
-// What a refill needs to know about a segment, cached in shared memory.
-struct IssueInfo {
-  int z0, nz, dir, ylo, N, rows, pad0, pad1;
-  const void* src[2][MAX_ARR];  // by buffer parity
+// A segment of the CTA as the passes use it, cached in shared memory (the inter-pass
+// waits drop L1, so a global read would miss it in every pass).
+struct alignas(16) SegInfo {
+  int z0, nz, dir, ylo, N, rows;  // rows: the tile's and one halo row on each side
+  int slot, flush, run, lat;      // run: the CTA's run on a lattice it belongs to
+  int slot_begin, slot_end;       // the lattice's slots
+  long long V;
+  const void* src[2][MAX_ARR];    // the arrays, by buffer parity (in groups a * V values apart)
 };
 
 // Shared-memory layout behind the stage ring of a DK pass (byte offsets).
@@ -112,8 +118,24 @@ constexpr size_t SM_RELEASED = 64;                              // 8 release cou
 constexpr size_t SM_OFF = 128;                                  // MAX_SEG_PER_CTA + 1 plane offsets
 constexpr size_t SM_RED = (SM_OFF + 4 * (MAX_SEG_PER_CTA + 1) + 127) / 128 * 128;  // 33 x NQ doubles
 constexpr size_t SM_FLAG = SM_RED + 33 * NQ * 8;                // 4 ints + pending tails
-constexpr size_t SM_INFO = (SM_FLAG + 16 + 4 * MAX_SEG_PER_CTA + 127) / 128 * 128;  // IssueInfo[]
-constexpr size_t SM_TAIL_BYTES = SM_INFO + MAX_SEG_PER_CTA * sizeof(IssueInfo);
+constexpr size_t SM_INFO = (SM_FLAG + 16 + 4 * MAX_SEG_PER_CTA + 127) / 128 * 128;  // SegInfo[nseg], records[nrun], TailPrep[min(nrun, 32)]
+
+// What the update of a lattice between two passes needs besides its sums, formed
+// before the wait for them (one per lane of the warp that runs the updates).
+struct TailPrep {
+  double wout, win, dnext;   // weights of the pass whose sums are taken
+  double ckn, dnn;           // kick weight and drift of the pass that starts
+  double pref, k[4];         // factors of the sums (the models' updates say which)
+  // fast (alpha = 1 with self-consistent expansion): b = a' after the two Friedmann kicks is
+  // b0 + c[0] s_kin + c[1] s_grad + c[2] s_pot of the pass's sums; a and pi2: the scale factor and sum of pi^2 before them
+  double b0, c[3], a, pi2;
+  int lat, fast;
+};
+// The bytes behind the stages for CTAs of at most nseg segments and nrun lattices,
+// whose records take run_bytes each.
+__host__ __device__ constexpr size_t sm_tail_bytes(int nseg, int nrun, size_t run_bytes) {
+  return SM_INFO + nseg * sizeof(SegInfo) + nrun * run_bytes + (nrun < 32 ? nrun : 32) * sizeof(TailPrep);
+}
 
 // Kick/drift weights of one pass (see the schedule in capi.cu).
 struct PassStep {
@@ -125,16 +147,18 @@ struct PassArgs {
   LatScalars* sc;
   const Seg* segs;
   const int* cta_seg;        // [gridDim.x + 1]
-  double* partials;          // [NQ][nslot]: quantity-major, so a lattice's slots are contiguous
+  double* partials;          // [2][NQ][nslot]: by the parity of the pass within the launch, then
+                             // quantity-major, so a lattice's slots are contiguous
   unsigned* counters;        // [nlat]
   double ck, wout, win, dnext;
   int parity, write, set_rho0, stages;
   unsigned stage_bytes_max;  // bytes of one stage (max over lattices)
   int nlat;                  // lattices advanced by the launch
   int nslot;                 // partial-sum slots of the launch (all lattices)
+  int nseg_max, nrun_max;    // segments, lattices of the CTA that has most of them
   unsigned long long wait_limit_ns;  // bound of every wait
-  // several passes in one cooperative launch (npass > 1): weights per pass and
-  // two monotonic counters (writes arrived, tails done), zeroed before launch
+  // several passes in one cooperative launch (npass > 1): weights per pass and a
+  // monotonic counter of the CTAs done with a pass, zeroed before launch
   const PassStep* steps;
   int npass, pad2;
   unsigned* gsync;
@@ -194,6 +218,12 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// One more on a counter that other CTAs read with ld_acquire_u32: everything this
+// thread has seen (its CTA's writes, after a block barrier) comes before it.
+__device__ __forceinline__ void red_release_inc(unsigned* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -250,7 +280,7 @@ __device__ __forceinline__ bool wait_counter(const unsigned* c, unsigned target,
   if ((int)(ld_acquire_u32(c) - target) >= 0) return true;
   const unsigned long long t0 = global_ns();
   for (uint32_t i = 0; i < (1u << 30); ++i) {
-    __nanosleep(64);
+    __nanosleep(20);
     if ((int)(ld_acquire_u32(c) - target) >= 0) return true;
     if ((i & 15u) == 15u && global_ns() - t0 > limit_ns) return false;
   }
@@ -305,10 +335,17 @@ template <> struct Acc<double> {
   __device__ __forceinline__ double value() const { return s; }
 };
 
-// Warp sum of one accumulator, returned on lane 0.  FP32 storage: the
-// (sum, -compensation) pairs of the lanes are combined pairwise with TwoSum
-// in FP32 and converted to FP64 once; FP64 storage: plain FP64 tree.
-__device__ __forceinline__ double warp_sum(const Acc<float>& a) {
+// Warp sum of one accumulator, on lane 0, as what the CTA's reduction keeps of a
+// warp (WarpPart): FP32 storage the (sum, compensation) pair, the lanes' (sum,
+// -compensation) pairs combined with TwoSum in FP32 (to be converted to FP64 once,
+// one lane per warp: every FP64 operation costs its warp 64 cycles however few
+// lanes take part); FP64 storage the sum of a plain FP64 tree.
+template <typename T> struct WarpPart;
+template <> struct WarpPart<float> { float hi, lo; };
+template <> struct WarpPart<double> { double v; };
+__device__ __forceinline__ double part_value(const WarpPart<float>& p) { return (double)p.hi + (double)p.lo; }
+__device__ __forceinline__ double part_value(const WarpPart<double>& p) { return p.v; }
+__device__ __forceinline__ WarpPart<float> warp_part(const Acc<float>& a) {
   float hi = a.s, lo = -a.c;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -319,14 +356,16 @@ __device__ __forceinline__ double warp_sum(const Acc<float>& a) {
     hi = s;
     lo = lo + l2 + e;
   }
-  return (double)hi + (double)lo;
+  return WarpPart<float>{hi, lo};
 }
-__device__ __forceinline__ double warp_sum(const Acc<double>& a) {
+__device__ __forceinline__ WarpPart<double> warp_part(const Acc<double>& a) {
   double v = a.s;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
+  return WarpPart<double>{v};
 }
+template <typename T>
+__device__ __forceinline__ double warp_sum(const Acc<T>& a) { return part_value(warp_part(a)); }
 
 // Fixed-order FP64 sum of part[begin .. end) over one warp (result on every
 // lane): lane l adds slots begin + l, + 32, ..., all of its first eight loads
@@ -340,9 +379,10 @@ __device__ __forceinline__ double warp_slot_sum(const double* part, int begin, i
     const int k = begin + lane + 32 * i;
     v[i] = k < end ? __ldcg(part + k) : 0.0;
   }
-  double s = 0.0;
+  double s = v[0];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) s += v[i];
+  for (int i = 1; i < 8; ++i)
+    if (begin + 32 * i < end) s += v[i];  // the same for the whole warp: an FP64 add costs it 64 cycles
   for (int k = begin + lane + 256; k < end; k += 32) s += __ldcg(part + k);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

@@ -11,10 +11,8 @@ namespace clg {
 // fixed power-law background): the drift over [eta, eta + dn] at the mean of
 // a(eta) and a(eta + dn), the values the deferred form computes in the tail of
 // the pass before.
-__device__ inline void kd_drift_coefficients(const LatConst& L, const LatScalars* SC, double dn, double& cd,
+__device__ inline void kd_drift_coefficients(const LatPar& L, const ScalarState& W, double dn, double& cd,
                                              double& cdA) {
-  ScalarState W;
-  load_state_cg(W, SC);
   const double an = L.expansion == CL_EXP_FIXED ? a_fixed(L, W, W.eta + dn) : W.a;
   drift_coefficients(L, 0.5 * (W.a + an), dn, cd, cdA);
 }

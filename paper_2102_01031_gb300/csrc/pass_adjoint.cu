@@ -85,10 +85,68 @@ __device__ __forceinline__ void st_v(T* p, const T (&v)[VX]) {
   *reinterpret_cast<typename V16<T>::type*>(p) = *reinterpret_cast<const typename V16<T>::type*>(v);
 }
 
+// dJ/dq and the adjoints of a and b after a reversed pass, and the coefficients of the
+// next (ring_pass_begin, ring_pass_end).
+template <typename T, bool SELF>
+struct AdjUpdate {
+  struct alignas(16) Rec {
+    double q, a, b, al, lq;                // dJ/dq so far, lam_a, lam_b; alpha and q
+    double c[ADJ_COEF_W], n[ADJ_COEF_W];   // coefficients of the pass whose sums are taken, and of the next
+    T cf[8];                               // cd, A1, A3, q, and lam_b times g_post, g_pre, g_phi, g_V
+  };
+  __device__ __forceinline__ static void load(const PassArgs& P, int lat, Rec* r) { get(&P.lat[lat], &P.sc[lat], r); }
+  __device__ __noinline__ static void get(const LatConst* L, const LatScalars* sc, Rec* r) {
+    r->q = __ldcg(&sc->adjq);
+    r->a = __ldcg(&sc->adja);
+    r->b = __ldcg(&sc->adjb);
+    r->al = L->alpha;
+    r->lq = L->q;
+  }
+  __device__ __forceinline__ static void ready(const PassArgs& P, int done, int next, Rec* r, TailPrep* q) {
+    q->fast = 0;
+    shift(P.adj + ADJ_COEF_W * next, done >= 0, next >= 0, r);
+  }
+  __device__ __noinline__ static void shift(const double* coef, bool done, bool next, Rec* r) {
+    for (int k = 0; k < ADJ_COEF_W; ++k) {
+      if (done) r->c[k] = r->n[k];
+      if (next) r->n[k] = __ldg(coef + k);
+    }
+  }
+  __device__ __forceinline__ static void fast_drift(Rec*, const TailPrep*, const double*) {}
+  __device__ __forceinline__ static void fast_powers(Rec*, const TailPrep*, const double*, double*, double*) {}
+  __device__ __noinline__ static void update(Rec* r, const TailPrep*, const double* Q, double*, cl_energies_t*, int) {
+    r->q += Q[0];
+    if (SELF) {
+      const double lak =
+          r->a + r->b * r->c[9] + ((1.0 + r->al) * r->c[2] * Q[1] - (3.0 + r->al) * r->c[3] * Q[2]) * r->c[8];
+      const double cq = Q[3] * r->c[10], w = r->c[11];
+      r->a = lak + cq;
+      r->b = r->b + w * lak + 0.5 * w * cq;
+    }
+  }
+  __device__ __noinline__ static void coefficients(Rec* r, const TailPrep*, double*) {
+    r->cf[0] = (T)r->n[0];
+    r->cf[1] = (T)r->n[2];
+    r->cf[2] = (T)r->n[3];
+    r->cf[3] = (T)r->lq;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r->cf[4 + k] = SELF ? (T)(r->b * r->n[4 + k]) : T(0);
+  }
+  __device__ __forceinline__ static void store(const PassArgs& P, int lat, const Rec* r) {
+    P.sc[lat].adjq = r->q;
+    P.sc[lat].adja = r->a;
+    P.sc[lat].adjb = r->b;
+  }
+};
+
+static_assert(sizeof(AdjUpdate<float, true>::Rec) == (5 + 2 * ADJ_COEF_W) * 8 + 8 * 4 + 8 &&
+                  sizeof(AdjUpdate<double, true>::Rec) == (5 + 2 * ADJ_COEF_W) * 8 + 8 * 8 + 8,
+              "adj_record_bytes in capi.cu");
+
 }  // namespace
 
 template <typename T, int NF, bool SELF>
-__global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const PassArgs P) {
+__global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const __grid_constant__ PassArgs P) {
   constexpr int VX = V16<T>::n;
   constexpr int NA = 4 * NF;
   constexpr int LF = 2 * NF;  // first adjoint array
@@ -98,48 +156,43 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const PassArgs P) 
   const Ring R = ring_view(smem, P);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sb = P.cta_seg[blockIdx.x], ns = P.cta_seg[blockIdx.x + 1] - sb;
-  const bool multi = P.npass > 1;
   if (tid == 0) ring_setup<NA>(R, P, sb, ns);
   __syncthreads();
   const int ptot = R.off[ns];
   const int S = R.S;
+  typedef AdjUpdate<T, SELF> Update;
+  const typename Update::Rec* const rec = reinterpret_cast<const typename Update::Rec*>(R.runs);
 
   int s_cur = 0;
   uint32_t p_cur = 0u;
   Acc<T> acc[NACC];
   float nonfinite = 0.f;
+  int fbuf = 0;
 #pragma unroll
   for (int k = 0; k < NACC; ++k) acc[k].zero();
 
   for (int pass = 0; pass < P.npass; ++pass) {
     const int parity = P.parity ^ (pass & 1);
-    const double* cfp = P.adj + ADJ_COEF_W * pass;
-    if (warp == 0) ring_pass_start<T, NA>(R, P, pass, ptot, parity, lane);
-    __syncthreads();
-    if (R.flag[0]) goto timeout;
+    if (!ring_pass_begin<T, NA, false, NACC, Update>(R, P, pass, ns, ptot, parity, false, warp, lane)) goto timeout;
 
     for (int i = 0; i < ns; ++i) {
-      const Seg sg = P.segs[sb + i];
-      const LatConst& L = P.lat[sg.lat];
-      const int N = L.N, BY = L.BY, TX = N / VX;
+      const SegInfo& si = R.info[i];
+      const int N = si.N, BY = si.rows - 2, TX = N / VX;
       const int tx = tid % TX, ty = tid / TX;
       const bool active = ty < BY;
       const int x0 = tx * VX;
-      const int y = sg.ytile * BY + ty;
+      const int y = si.ylo + ty;
       const int ae = (BY + 2) * N;
       const long long NN = (long long)N * N;
       const int g0 = R.off[i];
-      const T cd = (T)__ldg(cfp), A1 = (T)__ldg(cfp + 2), A3 = (T)__ldg(cfp + 3);
-      const T q = (T)L.q;
+      const T* const cf = rec[si.run].cf;
+      const T cd = cf[0], A1 = cf[1], A3 = cf[2], q = cf[3];
       // lam_b-scaled Friedmann-kick coefficients (lam_b is set by the previous reversed pass)
-      T bpost = T(0), bpre = T(0), bphi = T(0), bV = T(0);
-      if (SELF) {
-        const double lb = __ldcg(&P.sc[sg.lat].adjb);
-        bpost = (T)(lb * __ldg(cfp + 4));
-        bpre = (T)(lb * __ldg(cfp + 5));
-        bphi = (T)(lb * __ldg(cfp + 6));
-        bV = (T)(lb * __ldg(cfp + 7));
-      }
+      const T bpost = cf[4], bpre = cf[5], bphi = cf[6], bV = cf[7];
+      const int z0 = si.z0, nz = si.nz, dir = si.dir;
+      const long long Vs = si.V;
+      T* const out_s = static_cast<T*>(const_cast<void*>(si.src[parity ^ 1][0]));  // state, then adjoint
+      T* const out_l = static_cast<T*>(const_cast<void*>(si.src[parity ^ 1][LF]));
       const int xl = x0 == 0 ? N - 1 : x0 - 1, xr = x0 + VX == N ? 0 : x0 + VX;
       const int own = (ty + 1) * N + x0;
 
@@ -168,7 +221,7 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const PassArgs P) 
       uint32_t p_nxt = p_cur;
       ring_advance(S, s_nxt, p_nxt);
 
-      for (int j = 1; j <= sg.nz; ++j) {
+      for (int j = 1; j <= nz; ++j) {
         ring_wait(R, s_nxt, p_nxt, P.wait_limit_ns);
         if (active && !R.flag[0]) {
           const T* sa = ring_stage<T>(R, s_nxt);
@@ -254,13 +307,13 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const PassArgs P) 
             acc[3].add(s3);
           }
           const long long gi =
-              (long long)(sg.dir > 0 ? sg.z0 - 1 + j : sg.z0 + sg.nz - j) * NN + (long long)y * N + x0;
+              (long long)(dir > 0 ? z0 - 1 + j : z0 + nz - j) * NN + (long long)y * N + x0;
 #pragma unroll
           for (int k = 0; k < NF; ++k) {
-            st_v<T, VX>(reinterpret_cast<T*>(L.buf[parity ^ 1][2 * k]) + gi, nphi[k]);
-            st_v<T, VX>(reinterpret_cast<T*>(L.buf[parity ^ 1][2 * k + 1]) + gi, npi[k]);
-            st_v<T, VX>(reinterpret_cast<T*>(L.buf[parity ^ 1][LF + 2 * k]) + gi, nlf[k]);
-            st_v<T, VX>(reinterpret_cast<T*>(L.buf[parity ^ 1][LF + 2 * k + 1]) + gi, nlp[k]);
+            st_v<T, VX>(out_s + (2 * k) * Vs + gi, nphi[k]);
+            st_v<T, VX>(out_s + (2 * k + 1) * Vs + gi, npi[k]);
+            st_v<T, VX>(out_l + (2 * k) * Vs + gi, nlf[k]);
+            st_v<T, VX>(out_l + (2 * k + 1) * Vs + gi, nlp[k]);
           }
 #pragma unroll
           for (int k = 0; k < NF; ++k)
@@ -277,48 +330,15 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const PassArgs P) 
         p_cur = p_nxt;
         ring_advance(S, s_nxt, p_nxt);
       }
-      ring_release<T, NA>(R, g0 + sg.nz + 1, s_cur, parity, ptot, lane);
+      ring_release<T, NA>(R, g0 + nz + 1, s_cur, parity, ptot, lane);
       ring_advance(S, s_cur, p_cur);
 
-      if (!sg.flush) continue;
-      if (!ring_flush<NACC, NACC>(R, P, sg, acc, nonfinite, warp, lane)) goto timeout;
+      if (!si.flush) continue;
+      double* rb = R.red + fbuf * CONSUMER_WARPS * NQ;
+      fbuf ^= 1;
+      if (!ring_flush<NACC, NACC>(R, P, si, pass, acc, nonfinite, rb, (TX * BY + 31) >> 5, warp, lane)) goto timeout;
     }
-
-    // ---- end of the pass: all writes done; the lattice's dJ/dq share and scale-factor adjoints ----
-    if (multi && tid == 0) {
-      __threadfence();
-      fence_proxy_async_global();
-      atomicAdd(&P.gsync[0], 1u);
-    }
-    {
-      const int npend = R.flag[3];
-      for (int k = 0; k < npend; ++k) {
-        __threadfence();
-        const int lat = R.pend[k];
-        const LatConst& L = P.lat[lat];
-        ring_slot_sums<NACC>(R, P, L, warp, lane);
-        if (tid == 0) {
-          const double* Q = R.red + 32 * NQ;
-          LatScalars& Sc = P.sc[lat];
-          Sc.adjq = __ldcg(&Sc.adjq) + Q[0];
-          if (SELF) {
-            const double al = L.alpha, A1d = cfp[2], A3d = cfp[3];
-            const double la = __ldcg(&Sc.adja), lb = __ldcg(&Sc.adjb);
-            const double lak =
-                la + lb * cfp[9] + ((1.0 + al) * A1d * Q[1] - (3.0 + al) * A3d * Q[2]) * cfp[8];
-            const double cq = Q[3] * cfp[10], w = cfp[11];
-            Sc.adja = lak + cq;
-            Sc.adjb = lb + w * lak + 0.5 * w * cq;
-          }
-          P.counters[lat] = 0u;
-          __threadfence();
-          if (multi) atomicAdd(&P.gsync[1], 1u);
-        }
-        __syncthreads();
-      }
-      __syncthreads();
-      if (tid == 0) R.flag[3] = 0;
-    }
+    ring_pass_end<NACC, Update>(R, P, pass, ns, warp, lane);
   }
   return;
 
@@ -327,14 +347,14 @@ timeout:
   __syncthreads();
 }
 
-template __global__ void adj_pass_scalar<float, 1, false>(const PassArgs);
-template __global__ void adj_pass_scalar<float, 2, false>(const PassArgs);
-template __global__ void adj_pass_scalar<double, 1, false>(const PassArgs);
-template __global__ void adj_pass_scalar<double, 2, false>(const PassArgs);
-template __global__ void adj_pass_scalar<float, 1, true>(const PassArgs);
-template __global__ void adj_pass_scalar<float, 2, true>(const PassArgs);
-template __global__ void adj_pass_scalar<double, 1, true>(const PassArgs);
-template __global__ void adj_pass_scalar<double, 2, true>(const PassArgs);
+template __global__ void adj_pass_scalar<float, 1, false>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<float, 2, false>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<double, 1, false>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<double, 2, false>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<float, 1, true>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<float, 2, true>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<double, 1, true>(const __grid_constant__ PassArgs);
+template __global__ void adj_pass_scalar<double, 2, true>(const __grid_constant__ PassArgs);
 
 typedef void (*PassKernel)(const PassArgs);
 

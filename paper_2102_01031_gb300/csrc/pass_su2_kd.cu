@@ -230,7 +230,9 @@ __global__ void __launch_bounds__(TX * TY, (RED == 2 || sizeof(T) == 8) ? 1 : 20
     const LatScalars* SC = P.sc;
     const double ck = P.ck, ap1 = __ldcg(&SC->apow1), apm1 = __ldcg(&SC->apowm1), dx = L.dx;
     double kd, kdA;  // this pass's drift, after its kick
-    kd_drift_coefficients(L, SC, P.dnext, kd, kdA);
+    ScalarState W;
+    load_state_cg(W, SC);
+    kd_drift_coefficients(L, W, P.dnext, kd, kdA);
     cf[0] = (T)kd;
     cf[1] = (T)kdA;
     cf[2] = (T)(0.5 * L.gQB * dx * kdA);                         // half the SU(2) drift angle per momentum

@@ -123,6 +123,116 @@ __device__ __forceinline__ V plaq(V gd, V ai_n, V aj_npi, V ai_npj, V aj_n) {
   return vmul(gd, vsub(vadd(ai_n, aj_npi), vadd(ai_npj, aj_n)));
 }
 
+// The Friedmann update of a lattice between two passes and its coefficients in the
+// next (ring_pass_begin, ring_pass_end).
+template <typename T, int RED, bool KD>
+struct U1Update {
+  // cf: drift of fields and links (KD: after the kick, else deferred), kick coefficients
+  // of the covariant Laplacian, potential, current and curl, then gQ dx, v^2, lam
+  typedef LatRun<T, 9> Rec;
+
+  __device__ __forceinline__ static void load(const PassArgs& P, int lat, Rec* r) {
+    load_run(&P.lat[lat], &P.sc[lat], r);
+    r->cf[6] = (T)r->L.u1_gd;
+    r->cf[7] = (T)(r->L.v * r->L.v);
+    r->cf[8] = (T)r->L.lam;
+  }
+  __device__ __forceinline__ static void ready(const PassArgs& P, int done, int next, Rec* r, TailPrep* q) {
+    pass_weights_of(P.steps, PassStep{P.ck, P.wout, P.win, P.dnext}, done, next, q);
+    if (done >= 0) prepare(r, q);
+  }
+  // k: E_K per sum of pi_c^2, E_G per sum |D+ phi|^2, E_K^A per sum pi_A^2, E_G^A per sum (1 - cos)
+  __device__ __noinline__ static void prepare(const Rec* r, TailPrep* q) {
+    q->fast = 0;
+    if (RED == 0) return;
+    const LatPar& L = r->L;
+    if (RED == 1 && L.expansion == CL_EXP_SELF && L.int_alpha && L.alpha_i == 1) {
+      alpha1_ready(L, r->W, q);  // the links' energies enter with alpha - 1 = 0
+      return;
+    }
+    const double a = r->W.a, a2 = a * a, a4 = a2 * a2, a6 = a4 * a2;
+    const double gdx2 = L.gQ * L.dx * L.dx;
+    q->k[0] = 0.5 * L.inv_V / a6;
+    q->k[1] = 0.5 * L.inv_V * L.inv_dx2 / a2;
+    q->k[2] = 0.5 * L.inv_V / (L.fo2 * a4);
+    q->k[3] = L.inv_V / (L.fo2 * a4 * gdx2 * gdx2);
+    if (L.expansion == CL_EXP_SELF) q->pref = kernel_a_pref(L, a);
+  }
+  __device__ __noinline__ static void fast_drift(Rec* r, const TailPrep* q, const double* sum) {
+    alpha1_drift(r->W, q, alpha1_b(q, sum[0], sum[2], sum[4]));
+    r->cf[0] = (T)r->W.cd;
+    r->cf[1] = (T)r->W.cdA;
+    r->W.pi2 = sum[0];
+    r->W.pi2A = sum[1];
+  }
+  __device__ __noinline__ static void fast_powers(Rec* r, const TailPrep* q, const double* sum, double*, double*) {
+    alpha1_powers(r->W, q, alpha1_b(q, sum[0], sum[2], sum[4]));
+    const double k1 = q->ckn * r->W.apow1;
+    r->cf[2] = (T)(k1 * r->L.inv_dx2);
+    r->cf[3] = (T)(q->ckn * r->W.apow3);
+    r->cf[4] = (T)(k1 * r->L.u1_cJ);
+    r->cf[5] = (T)(-q->ckn * r->W.apowm1 * r->L.u1_cC);
+  }
+  __device__ __noinline__ static void update(Rec* r, const TailPrep* q, const double* sum, double*, cl_energies_t* ob,
+                                             int set_rho0) {
+    const LatPar& L = r->L;
+    const PassStep st = {0.0, q->wout, q->win, q->dnext};
+    ScalarState W = r->W;
+    PassSums E = {0, 0, 0, 0, 0, 0, 0};
+    if (RED > 0) {
+      constexpr int o = RED == 1 ? 0 : 1;
+      const double spost = RED == 1 ? sum[0] : sum[0] + sum[1];
+      const double spA = sum[1 + o], gg = sum[2 + o], mag = sum[3 + o], vs = sum[4 + o];
+      E.EKpre = W.pi2 * q->k[0];
+      E.EKpost = spost * q->k[0];
+      E.EKApre = W.pi2A * q->k[2];
+      E.EKA = spA * q->k[2];
+      E.EG = gg * q->k[1];
+      E.EGA = mag * q->k[3];
+      E.EV = vs * L.inv_V;
+      W.pi2 = spost;
+      W.pi2A = spA;
+      if (L.expansion == CL_EXP_SELF) advance_scalars(st, L, W, E, true, q->pref);
+    }
+    if (RED == 2 && ob) {
+      for (int k2 = 0; k2 < 4; ++k2) {
+        ob->EK[k2] = ob->EG[k2] = ob->EV[k2] = 0.0;
+        ob->mean_phi[k2] = ob->mean_phi2[k2] = ob->mean_pi[k2] = ob->mean_pi2[k2] = 0.0;
+      }
+      ob->EK[0] = E.EKpost;
+      ob->EG[0] = E.EG;
+      ob->EV[0] = E.EV;
+      ob->EKA = E.EKA;
+      ob->EGA = E.EGA;
+      for (int c = 0; c < 2; ++c) {
+        ob->mean_phi[c] = sum[6 + c] * L.inv_V;
+        ob->mean_phi2[c] = sum[8 + c] * L.inv_V;
+        ob->mean_pi[c] = sum[10 + c] * L.inv_V;
+        ob->mean_pi2[c] = sum[c] * L.inv_V;
+      }
+      ob->nonfinite = (int64_t)sum[NQ - 1];
+      finish_obs(set_rho0, L, W, *ob);
+    }
+    advance_drift(st.dnext, L, W);
+    r->W = W;
+  }
+  __device__ __noinline__ static void coefficients(Rec* r, const TailPrep* q, double*) {
+    const ScalarState& W = r->W;
+    const LatPar& L = r->L;
+    double cd = W.cd, cdA = W.cdA;
+    if (KD) kd_drift_coefficients(L, W, q->dnn, cd, cdA);
+    r->cf[0] = (T)cd;
+    r->cf[1] = (T)cdA;
+    const double k1 = q->ckn * W.apow1;
+    r->cf[2] = (T)(k1 * L.inv_dx2);
+    r->cf[3] = (T)(q->ckn * W.apow3);
+    r->cf[4] = (T)(k1 * L.u1_cJ);  // (2 gQ/dx) Im[...] = (gQ/dx)(phi_0 u_1 - phi_1 u_0)
+    r->cf[5] = (T)(-q->ckn * W.apowm1 * L.u1_cC);
+  }
+  __device__ __forceinline__ static void store(const PassArgs& P, int lat, const Rec* r) { put(&P.sc[lat], r); }
+  __device__ __noinline__ static void put(LatScalars* to, const Rec* r) { store_state(to, r->W); }
+};
+
 }  // namespace
 
 // RED: 0 = no sums, 1 = sums for the Friedmann kick, 2 = full measurement.
@@ -138,7 +248,7 @@ __device__ __forceinline__ V plaq(V gd, V ai_n, V aj_npi, V ai_npj, V aj_n) {
 // kernel is built for N = NC with full tiles of THREADS threads (every stage
 // offset a compile-time constant).
 template <typename T, int RED, bool KD, int NC>
-__global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const PassArgs P) {
+__global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__ PassArgs P) {
   constexpr int VX = U1Vec<T>::n;
   typedef typename U1Vec<T>::type V;
   constexpr int NAR = 10;  // arrays in a ring stage
@@ -151,76 +261,49 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const PassArgs P) {
   const Ring R = ring_view(smem, P);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sb = P.cta_seg[blockIdx.x], ns = P.cta_seg[blockIdx.x + 1] - sb;
-  const bool multi = P.npass > 1;
   if (tid == 0) ring_setup<NAR>(R, P, sb, ns);
   __syncthreads();
   const int ptot = R.off[ns];
   const int S = R.S;
+  typedef U1Update<T, RED, KD> Update;
+  const typename Update::Rec* const rec = reinterpret_cast<const typename Update::Rec*>(R.runs);
 
   int s_cur = 0;
   uint32_t p_cur = 0u;
   Acc<T> acc[NACC];
   float nonfinite = 0.f;
+  int fbuf = 0;
 #pragma unroll
   for (int k = 0; k < NACC; ++k) acc[k].zero();
 
   for (int pass = 0; pass < P.npass; ++pass) {
     const int parity = P.parity ^ (pass & 1);
-    if (warp == 0) ring_pass_start<T, NAR, KD>(R, P, pass, ptot, parity, lane);
-    __syncthreads();
-    if (R.flag[0]) goto timeout;
+    if (!ring_pass_begin<T, NAR, KD, NUSED, Update>(R, P, pass, ns, ptot, parity, false, warp, lane)) goto timeout;
 
     for (int i = 0; i < ns; ++i) {
-      const Seg sg = P.segs[sb + i];
-      const LatConst& L = P.lat[sg.lat];
-      const int N = NC ? NC : L.N, BY = NC ? THREADS / (NC / VX) : L.BY, TX = N / VX;
+      const SegInfo& si = R.info[i];
+      const int N = NC ? NC : si.N, BY = NC ? THREADS / (NC / VX) : si.rows - 2, TX = N / VX;
       const int tx = tid % TX, ty = tid / TX;
       const bool active = ty < BY;  // threads 0 .. TX*BY-1
       const int x0 = tx * VX;
-      const int y = sg.ytile * BY + ty;
+      const int y = si.ylo + ty;
       const int ae = (BY + 2) * N;  // elements of one array in a stage
       // stage offset of array a: KD keeps (field, momentum) pairs of BY + 2 and BY rows
       auto aoff = [&](int a) { return KD ? (a >> 1) * (2 * BY + 2) * N + (a & 1) * ae : a * ae; };
       const int mrow = KD ? -N : 0;  // KD: a momentum's stage rows start at the tile's first row
       const long long NN = (long long)N * N;
       const int g0 = R.off[i];
-      // coefficients of the segment: FP64 products formed by one lane (the
-      // FP64 pipe is narrow) and broadcast in the storage precision
-      T cf[10];
-      if (lane == 0) {
-        const LatScalars* SC = &P.sc[sg.lat];
-        const double ckp = P.steps ? __ldg(&P.steps[pass].ck) : P.ck;
-        const double ap1 = __ldcg(&SC->apow1);
-        if constexpr (KD) {
-          // no deferred drift to apply on read; this pass's drift, after its kick
-          double kd, kdA;
-          kd_drift_coefficients(L, SC, P.steps ? __ldg(&P.steps[pass].dnext) : P.dnext, kd, kdA);
-          cf[0] = cf[1] = T(0);
-          cf[8] = (T)kd;
-          cf[9] = (T)kdA;
-        } else {
-          cf[0] = (T)__ldcg(&SC->cd);
-          cf[1] = (T)__ldcg(&SC->cdA);
-          cf[8] = cf[9] = T(0);
-        }
-        cf[2] = (T)(ckp * ap1 * L.inv_dx2);
-        cf[3] = (T)(ckp * __ldcg(&SC->apow3));
-        cf[4] = (T)(ckp * ap1 * L.u1_cJ);   // (2 gQ/dx) Im[...] = (gQ/dx)(phi_0 u_1 - phi_1 u_0)
-        cf[5] = (T)(-ckp * __ldcg(&SC->apowm1) * L.u1_cC);
-        cf[6] = (T)L.u1_gd;
-        cf[7] = (T)(L.v * L.v);
-      }
-#pragma unroll
-      for (int k = 0; k < 10; ++k) cf[k] = __shfl_sync(0xffffffffu, cf[k], 0);
-      const T cd = cf[0], cdA = cf[1], A1 = cf[2], A3 = cf[3], AJ = cf[4], AC = cf[5], gd = cf[6], v2 = cf[7];
-      const T kd = cf[8], kdA = cf[9];  // KD: the drift after the kick
+      const T* const cf = rec[si.run].cf;
+      const T A1 = cf[2], A3 = cf[3], AJ = cf[4], AC = cf[5], gd = cf[6], v2 = cf[7], lam = cf[8];
+      // KD: no deferred drift to apply on read, this pass's drift after its kick
+      const T cd = KD ? T(0) : cf[0], cdA = KD ? T(0) : cf[1], kd = KD ? cf[0] : T(0), kdA = KD ? cf[1] : T(0);
       const bool drifting = !KD && (cd != T(0) || cdA != T(0));
-      const T lam = (T)L.lam;
       const V gdv = vset(gd);
       const int xl = x0 == 0 ? N - 1 : x0 - 1, xr = x0 + VX == N ? 0 : x0 + VX;
       // output buffer: array a of a lattice buffer starts a * V elements after array 0
-      T* const dbase = reinterpret_cast<T*>(L.buf[parity ^ 1][0]);
-      const long long Vs = L.V;
+      T* const dbase = static_cast<T*>(const_cast<void*>(si.src[parity ^ 1][0]));
+      const long long Vs = si.V;
+      const int z0 = si.z0, nz = si.nz;
 
       // the thread's sites of field array a (its momentum is a + 1) on stage row `row`, drifted
       auto rdv = [&](const T* st, int a, int row, T coef) -> V {
@@ -274,14 +357,14 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const PassArgs P) {
       uint32_t p_nxt = p_cur;
       ring_advance(S, s_nxt, p_nxt);
 
-      for (int j = 1; j <= sg.nz; ++j) {  // plane j in stage s_cur, plane j + 1 in s_nxt
+      for (int j = 1; j <= nz; ++j) {  // plane j in stage s_cur, plane j + 1 in s_nxt
         ring_wait(R, s_nxt, p_nxt, P.wait_limit_ns);
         if (active && !R.flag[0]) {
           const T* sa = ring_stage<T>(R, s_nxt);
           const T* sc = ring_stage<T>(R, s_cur);
           const int own = (ty + 1) * N + x0;
           // segments march up and never wrap: plane j is z0 + j - 1
-          T* const out = dbase + (long long)(sg.z0 + j - 1) * NN + (long long)y * N + x0;
+          T* const out = dbase + (long long)(z0 + j - 1) * NN + (long long)y * N + x0;
           const V aF0 = rdv(sa, F0, ty + 1, cd), aF1 = rdv(sa, F1, ty + 1, cd);  // plane above, drifted
           const V aA0 = rdv(sa, AX, ty + 1, cdA), aA1 = rdv(sa, AY, ty + 1, cdA);
           const V ay_ym = rdv(sc, AY, ty, cdA), ay_ymzp = rdv(sa, AY, ty, cdA);
@@ -463,90 +546,15 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const PassArgs P) {
         p_cur = p_nxt;
         ring_advance(S, s_nxt, p_nxt);
       }
-      ring_release<T, NAR, KD>(R, g0 + sg.nz + 1, s_cur, parity, ptot, lane);
+      ring_release<T, NAR, KD>(R, g0 + nz + 1, s_cur, parity, ptot, lane);
       ring_advance(S, s_cur, p_cur);
 
-      if (!sg.flush) continue;
-      if (!ring_flush<NACC, NUSED>(R, P, sg, acc, nonfinite, warp, lane)) goto timeout;
+      if (!si.flush) continue;
+      double* rb = R.red + fbuf * CONSUMER_WARPS * NQ;
+      fbuf ^= 1;
+      if (!ring_flush<NACC, NUSED>(R, P, si, pass, acc, nonfinite, rb, (TX * BY + 31) >> 5, warp, lane)) goto timeout;
     }
-
-    // ---- end of the pass ----
-    if (multi && tid == 0) {  // this CTA's writes are done
-      __threadfence();
-      fence_proxy_async_global();
-      atomicAdd(&P.gsync[0], 1u);
-    }
-    {
-      const int npend = R.flag[3];
-      const PassStep pst = P.steps ? P.steps[pass] : PassStep{P.ck, P.wout, P.win, P.dnext};
-      for (int k = 0; k < npend; ++k) {
-        __threadfence();
-        const int lat = R.pend[k];
-        const LatConst& L = P.lat[lat];
-        ring_slot_sums<NUSED>(R, P, L, warp, lane);
-        if (tid == 0) {
-          PassArgs Q = P;
-          Q.ck = pst.ck;
-          Q.wout = pst.wout;
-          Q.win = pst.win;
-          Q.dnext = pst.dnext;
-          ScalarState W;
-          load_state_cg(W, &P.sc[lat]);
-          const double* sum = R.red + 32 * NQ;
-          const double a = W.a, a2 = a * a, a4 = a2 * a2, a6 = a4 * a2;
-          const double gdx2 = L.gQ * L.dx * L.dx;
-          const double kphi = 0.5 * L.inv_V / a6;                       // E_K per sum of pi_c^2
-          const double gphi = 0.5 * L.inv_V * L.inv_dx2 / a2;           // E_G per sum |D+ phi|^2
-          const double kA = 0.5 * L.inv_V / (L.fo2 * a4);               // E_K^A per sum pi_A^2
-          const double mA = L.inv_V / (L.fo2 * a4 * gdx2 * gdx2);       // E_G^A per sum (1 - cos)
-          PassSums E = {0, 0, 0, 0, 0, 0, 0};
-          double spost = 0.0;
-          if (RED > 0) {
-            constexpr int o = RED == 1 ? 0 : 1;
-            spost = RED == 1 ? sum[0] : sum[0] + sum[1];
-            const double spA = sum[1 + o], gg = sum[2 + o], mag = sum[3 + o], vs = sum[4 + o];
-            E.EKpre = W.pi2 * kphi;
-            E.EKpost = spost * kphi;
-            E.EKApre = W.pi2A * kA;
-            E.EKA = spA * kA;
-            E.EG = gg * gphi;
-            E.EGA = mag * mA;
-            E.EV = vs * L.inv_V;
-            W.pi2 = spost;
-            W.pi2A = spA;
-          }
-          advance_scalars(Q, L, W, E, RED > 0);
-          if (RED == 2) {
-            cl_energies_t& ob = P.sc[lat].obs;
-            for (int k2 = 0; k2 < 4; ++k2) {
-              ob.EK[k2] = ob.EG[k2] = ob.EV[k2] = 0.0;
-              ob.mean_phi[k2] = ob.mean_phi2[k2] = ob.mean_pi[k2] = ob.mean_pi2[k2] = 0.0;
-            }
-            ob.EK[0] = E.EKpost;
-            ob.EG[0] = E.EG;
-            ob.EV[0] = E.EV;
-            ob.EKA = E.EKA;
-            ob.EGA = E.EGA;
-            for (int c = 0; c < 2; ++c) {
-              ob.mean_phi[c] = sum[6 + c] * L.inv_V;
-              ob.mean_phi2[c] = sum[8 + c] * L.inv_V;
-              ob.mean_pi[c] = sum[10 + c] * L.inv_V;
-              ob.mean_pi2[c] = sum[c] * L.inv_V;
-            }
-            ob.nonfinite = (int64_t)sum[NQ - 1];
-            finish_obs(Q, L, W, ob);
-          }
-          advance_drift(Q, L, W);
-          store_state(&P.sc[lat], W);
-          P.counters[lat] = 0u;
-          __threadfence();
-          if (multi) atomicAdd(&P.gsync[1], 1u);
-        }
-        __syncthreads();
-      }
-      __syncthreads();
-      if (tid == 0) R.flag[3] = 0;
-    }
+    ring_pass_end<NUSED, Update>(R, P, pass, ns, warp, lane);
   }
   return;
 
@@ -555,18 +563,18 @@ timeout:
   __syncthreads();
 }
 
-template __global__ void dk_pass_u1<float, 0, false, 0>(const PassArgs);
-template __global__ void dk_pass_u1<float, 1, false, 0>(const PassArgs);
-template __global__ void dk_pass_u1<float, 2, false, 0>(const PassArgs);
-template __global__ void dk_pass_u1<double, 0, false, 0>(const PassArgs);
-template __global__ void dk_pass_u1<double, 1, false, 0>(const PassArgs);
-template __global__ void dk_pass_u1<double, 2, false, 0>(const PassArgs);
-template __global__ void dk_pass_u1<float, 0, true, 0>(const PassArgs);
-template __global__ void dk_pass_u1<float, 2, true, 0>(const PassArgs);
-template __global__ void dk_pass_u1<double, 0, true, 0>(const PassArgs);
-template __global__ void dk_pass_u1<double, 2, true, 0>(const PassArgs);
-template __global__ void dk_pass_u1<float, 0, true, 256>(const PassArgs);
-template __global__ void dk_pass_u1<float, 2, true, 256>(const PassArgs);
+template __global__ void dk_pass_u1<float, 0, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, 1, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, 2, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<double, 0, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<double, 1, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<double, 2, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, 0, true, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, 2, true, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<double, 0, true, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<double, 2, true, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, 0, true, 256>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, 2, true, 256>(const __grid_constant__ PassArgs);
 
 typedef void (*PassKernel)(const PassArgs);
 

@@ -1,19 +1,44 @@
 // ring.cuh -- the plane ring of a DK pass, as device functions: the shared
 // memory behind the stages, the bulk copies that fill a stage with one z-plane
 // tile of every array, the release count whose last warp refills the stage,
-// the per-run flush of the sums into a partial-sum slot, and the lattice-wide
-// slot reduction that precedes the Friedmann update.
+// the per-run flush of the sums into a partial-sum slot, and what joins two
+// passes of one launch.
 //
 // A CTA's segments form one sequence of planes (each segment adds a halo
 // plane at both ends); plane g of pass p lives in stage (p * ptot + g) mod S.
 // A stage holds, for every array, the plane's BY rows of the segment's y-tile
 // plus one halo row on each side, each row complete in x (with MOWN the momenta,
 // read at the tile's own sites only, without the halo rows).
+//
+// Between two passes of a launch the whole lattice's sums decide the next scale
+// factor.  Every CTA keeps the scalars of the lattices it works on in shared
+// memory (LatRun) and runs their Friedmann update itself, from the slots all CTAs
+// wrote: one counter and one wait join the passes.  (The update used to be run by
+// the CTA that wrote a lattice's last slot, and a second counter told the others:
+// two more trips through L2 and the new scalars read back, with FP64 coefficients
+// formed by every warp.)  Two sets of slots alternate, since a CTA may write its
+// next sums while another still reads these; every CTA adds the same slots in the
+// same order, so all hold the same scalars.  The last pass of a launch leaves them
+// in global memory: there the CTA that completes a lattice's arrival count runs
+// the update and stores it.
 #pragma once
 
 #include "common.cuh"
+#include "tail.cuh"
 
 namespace clg {
+
+// A CTA's run on one lattice: the lattice's evolving scalars as of the current
+// pass, its constants, and the pass's coefficients in the storage precision.
+template <typename T, int NCF>
+struct alignas(16) LatRun {
+  ScalarState W;
+  LatPar L;
+  T cf[NCF];
+};
+static_assert(sizeof(LatRun<float, 4>) == (sizeof(ScalarState) + sizeof(LatPar) + 16 + 15) / 16 * 16 &&
+                  sizeof(LatRun<double, 9>) == (sizeof(ScalarState) + sizeof(LatPar) + 72 + 15) / 16 * 16,
+              "run_record_bytes in capi.cu");
 
 struct Ring {
   unsigned char* stages;  // S stages of stage_bytes
@@ -21,9 +46,10 @@ struct Ring {
   unsigned* released;     // warps done with each stage
   int* off;               // first plane of each segment, and the total
   double* red;            // [33][NQ] reduction scratch
-  volatile int* flag;     // [0] timed out, [1] unused, [2] lattice of the last run, [3] #pending tails
-  int* pend;              // lattices whose Friedmann update this CTA runs
-  IssueInfo* info;        // per segment: what its refills copy
+  volatile int* flag;     // [0] timed out, [1] runs of the CTA, [2] lattice of the last run, [3] #pending tails
+  int* pend;              // runs whose lattices' Friedmann update this CTA stores
+  SegInfo* info;          // per segment
+  unsigned char* runs;    // LatRun records
   int S;
   unsigned stage_bytes;
 };
@@ -40,12 +66,13 @@ __device__ __forceinline__ Ring ring_view(unsigned char* smem, const PassArgs& P
   R.red = reinterpret_cast<double*>(tail + SM_RED);
   R.flag = reinterpret_cast<volatile int*>(tail + SM_FLAG);
   R.pend = reinterpret_cast<int*>(tail + SM_FLAG + 16);
-  R.info = reinterpret_cast<IssueInfo*>(tail + SM_INFO);
+  R.info = reinterpret_cast<SegInfo*>(tail + SM_INFO);
+  R.runs = tail + SM_INFO + (size_t)P.nseg_max * sizeof(SegInfo);
   return R;
 }
 
-// Thread 0: barriers, counts, flags, plane offsets and the copy info of the
-// CTA's `ns` segments starting at segs[sb].
+// Thread 0: barriers, counts, flags, plane offsets and the records of the CTA's
+// `ns` segments starting at segs[sb].
 template <int NA>
 __device__ void ring_setup(const Ring& R, const PassArgs& P, int sb, int ns) {
   for (int s = 0; s < R.S; ++s) {
@@ -54,25 +81,56 @@ __device__ void ring_setup(const Ring& R, const PassArgs& P, int sb, int ns) {
   }
   fence_mbar_init();
   R.flag[0] = 0;
-  R.flag[1] = 0;
   R.flag[2] = ns > 0 ? P.segs[sb].lat : 0;
   R.flag[3] = 0;
   R.off[0] = 0;
+  int run = -1;
   for (int i = 0; i < ns; ++i) {
-    const Seg& sg = P.segs[sb + i];
+    const Seg sg = P.segs[sb + i];
     const LatConst& L = P.lat[sg.lat];
     R.off[i + 1] = R.off[i] + sg.nz + 2;
-    IssueInfo& in = R.info[i];
+    SegInfo& in = R.info[i];
+    if (i == 0 || R.info[i - 1].lat != sg.lat) ++run;
     in.z0 = sg.z0;
     in.nz = sg.nz;
     in.dir = sg.dir;
     in.ylo = sg.ytile * L.BY;
     in.N = L.N;
     in.rows = L.BY + 2;
-    for (int a = 0; a < NA; ++a) {
-      in.src[0][a] = L.buf[0][a];
-      in.src[1][a] = L.buf[1][a];
-    }
+    in.slot = sg.slot;
+    in.flush = sg.flush;
+    in.run = run;
+    in.lat = sg.lat;
+    in.slot_begin = L.slot_begin;
+    in.slot_end = L.slot_end;
+    in.V = L.V;
+    for (int p = 0; p < 2; ++p)
+      for (int a = 0; a < NA; ++a) in.src[p][a] = L.buf[p][a];
+  }
+  R.flag[1] = run + 1;
+}
+
+// A segment of run r of the CTA (its segments are grouped by lattice).
+__device__ __forceinline__ const SegInfo& ring_run(const Ring& R, int ns, int r) {
+  int i = 0;
+  while (i + 1 < ns && R.info[i].run != r) ++i;
+  return R.info[i];
+}
+
+// Sums of the first NUSED quantities of the lattices of the CTA's runs which(0) ..
+// which(nb - 1) into rows of red, the warps sharing the (lattice, quantity) pairs,
+// each over the lattice's slots in a fixed order (warp_slot_sum), so that the result
+// depends neither on timing nor on the CTA.
+template <int NUSED, class Which>
+__device__ __forceinline__ void ring_slot_sums(const Ring& R, const PassArgs& P, int pass, int ns, int nb, int warp,
+                                               int lane, Which which) {
+  constexpr int NQU = NUSED > 0 ? NUSED : 1;
+  const double* slots = P.partials + (size_t)(pass & 1) * NQ * P.nslot;
+  for (int it = CONSUMER_WARPS - 1 - warp; it < nb * NUSED; it += CONSUMER_WARPS) {
+    const int l = it / NQU, q = it - l * NQU;
+    const SegInfo& in = ring_run(R, ns, which(l));
+    const double s = warp_slot_sum(slots + (size_t)q * P.nslot, in.slot_begin, in.slot_end, lane);
+    if (lane == 0) R.red[l * NQ + q] = s;
   }
 }
 
@@ -81,7 +139,7 @@ __device__ __forceinline__ const T* ring_stage(const Ring& R, int s) {
   return reinterpret_cast<const T*>(R.stages + (size_t)s * R.stage_bytes);
 }
 
-// Bulk copies of plane g (of the current pass) into stage s, issued by a
+// Bulk copies of plane g (of the forward sequence) into stage s, issued by a
 // whole warp (warp-uniform call): lane a + NA k copies run k of array a (a
 // tile's rows form up to three runs where they wrap around the periodic y
 // boundary).  MOWN: the odd arrays (momenta of a field/momentum layout) are
@@ -95,7 +153,7 @@ __device__ void ring_issue_warp(const Ring& R, int g, int s, int parity, int lan
   static_assert(3 * NA <= 32, "one lane per copy");
   int i = 0;
   while (g >= R.off[i + 1]) ++i;
-  const IssueInfo& in = R.info[i];
+  const SegInfo& in = R.info[i];
   const int N = in.N, rows = in.rows, arr_elems = rows * N;
   const int j = g - R.off[i];
   int zp = in.dir > 0 ? in.z0 - 1 + j : in.z0 + in.nz - j;
@@ -127,8 +185,11 @@ __device__ void ring_issue_warp(const Ring& R, int g, int s, int parity, int lan
 
 // A warp is done with plane g (in stage s); the last of the CTA's warps
 // refills s with plane g + S of the same pass (which belongs in the same stage).
+// rev: the pass marches the CTA's sequence backwards (plane g is plane
+// ptot - 1 - g of the forward sequence).
 template <typename T, int NA, bool MOWN = false>
-__device__ __forceinline__ void ring_release(const Ring& R, int g, int s, int parity, int ptot, int lane) {
+__device__ __forceinline__ void ring_release(const Ring& R, int g, int s, int parity, int ptot, int lane,
+                                             bool rev = false) {
   __syncwarp();
   int refill = 0;
   if (lane == 0) {
@@ -139,7 +200,8 @@ __device__ __forceinline__ void ring_release(const Ring& R, int g, int s, int pa
       refill = g + R.S < ptot && !R.flag[0];
     }
   }
-  if (__shfl_sync(0xffffffffu, refill, 0)) ring_issue_warp<T, NA, MOWN>(R, g + R.S, s, parity, lane);
+  if (__shfl_sync(0xffffffffu, refill, 0))
+    ring_issue_warp<T, NA, MOWN>(R, rev ? ptot - 1 - (g + R.S) : g + R.S, s, parity, lane);
   __syncwarp();
 }
 
@@ -156,27 +218,42 @@ __device__ __forceinline__ void ring_advance(int S, int& s, uint32_t& p) {
   }
 }
 
+__device__ __forceinline__ bool last_pass(const PassArgs& P, int pass) { return pass + 1 >= P.npass; }
+
+// This pass's set of partial-sum slots.
+__device__ __forceinline__ double* pass_slots(const PassArgs& P, int pass) {
+  return P.partials + (size_t)(pass & 1) * NQ * P.nslot;
+}
+
 // End of a CTA's run on a lattice (all threads): warp partials of the NUSED
-// slots (accumulators acc[0..NACC), slot NQ-1 = non-finite count), a fixed
-// shuffle tree over the warps per slot into P.partials, and the lattice's
-// arrival count; the CTA that completes it queues the lattice's tail.
-// Returns false if a wait of this CTA had timed out.
+// slots (accumulators acc[0..NACC), slot NQ-1 = non-finite count) into rb, a fixed
+// shuffle tree over the warps per quantity into this pass's slots; in the last pass
+// also one arrival per quantity on the lattice's count, and the arrival that
+// completes it queues the lattice's update.  busy: warps that had any site (the
+// others' sums are zero and are not formed).  rb: one of two alternating halves of
+// red (a warp can reach the next flush while others still read this one, but not
+// the one after, which waits for all).  Returns false if a wait of this CTA had
+// timed out.
 template <int NACC, int NUSED, typename T>
-__device__ bool ring_flush(const Ring& R, const PassArgs& P, const Seg& sg, Acc<T> (&acc)[NACC],
-                           float& nonfinite, int warp, int lane) {
-  if (NUSED > 0) {
+__device__ __forceinline__ bool ring_flush(const Ring& R, const PassArgs& P, const SegInfo& sg, int pass,
+                                           Acc<T> (&acc)[NACC], float& nonfinite, double* red_half, int busy, int warp,
+                                           int lane) {
+  constexpr int NARRIVE = NUSED > 0 ? NUSED : 1;
+  static_assert(sizeof(WarpPart<T>) == sizeof(double), "a warp's part takes one entry of red");
+  WarpPart<T>* const rb = reinterpret_cast<WarpPart<T>*>(red_half);
+  if (NUSED > 0 && warp < busy) {
 #pragma unroll
     for (int k = 0; k < NUSED; ++k) {
-      double v = 0.0;
+      WarpPart<T> v = {};
       if (k < NACC) {
-        v = warp_sum(acc[k]);
+        v = warp_part(acc[k]);
       } else if (k == NQ - 1) {
         float c = nonfinite;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-        v = (double)c;
+        v = WarpPart<T>{c};
       }
-      if (lane == 0) R.red[warp * NQ + k] = v;
+      if (lane == 0) rb[warp * NQ + k] = v;
     }
   }
 #pragma unroll
@@ -184,60 +261,151 @@ __device__ bool ring_flush(const Ring& R, const PassArgs& P, const Seg& sg, Acc<
   nonfinite = 0.f;
   __syncthreads();
   if (R.flag[0]) return false;
-  if (warp < NUSED) {
-    double v = lane < CONSUMER_WARPS ? R.red[lane * NQ + warp] : 0.0;
+  const bool last = last_pass(P, pass);
+  if (warp < NARRIVE) {
+    double v = 0.0;
+    if (NUSED > 0) {
+      v = lane < busy ? part_value(rb[lane * NQ + warp]) : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      for (int o = CONSUMER_WARPS / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    }
     if (lane == 0) {
-      P.partials[(size_t)warp * P.nslot + sg.slot] = v;
-      __threadfence();
+      if (NUSED > 0) pass_slots(P, pass)[(size_t)warp * P.nslot + sg.slot] = v;
+      if (last) {
+        __threadfence();
+        const unsigned nslot = (unsigned)(sg.slot_end - sg.slot_begin);
+        const unsigned prev = atomicAdd(&P.counters[sg.lat], 1u);
+        if (prev == NARRIVE * nslot - 1u) R.pend[atomicAdd(const_cast<int*>(&R.flag[3]), 1)] = sg.run;
+      }
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const LatConst& L = P.lat[sg.lat];
-    const unsigned nslot = (unsigned)(L.slot_end - L.slot_begin);
-    const unsigned prev = atomicAdd(&P.counters[sg.lat], 1u);
-    R.flag[2] = sg.lat;
-    if (prev == nslot - 1u) R.pend[R.flag[3]++] = sg.lat;
-  }
-  __syncthreads();
+  if (threadIdx.x == 0) R.flag[2] = sg.lat;
   return true;
 }
 
-// Lattice-wide sums of the first NUSED quantities into red[32 * NQ + k]:
-// warp k sums the lattice's slots of quantity k in a fixed order
-// (warp_slot_sum), so the result does not depend on timing.  All threads;
-// ends with a barrier.
-template <int NUSED>
-__device__ void ring_slot_sums(const Ring& R, const PassArgs& P, const LatConst& L, int warp,
-                               int lane) {
-  if (warp < NUSED) {
-    const double s = warp_slot_sum(P.partials + (size_t)warp * P.nslot, L.slot_begin, L.slot_end, lane);
-    if (lane == 0) R.red[32 * NQ + warp] = s;
+// Joins pass - 1 and pass of a launch, or starts it (pass 0); all threads.  Waits
+// (bounded) until every CTA's writes of the previous pass are done, issues the
+// first planes of this pass, one warp per plane, and meanwhile brings the record of
+// every lattice of the CTA up to date, lane r mod 32 of the last warp for run r:
+//   U::load(P, lattice, record)             pass 0: constants and scalars from global memory;
+//   U::ready(P, done, next, record, prep)   before the wait: the weights of the pass whose sums are taken
+//                                           and of the next, and what does not depend on the sums;
+//   U::update(record, prep, sums, log of the last pass, ...)   with the previous pass's NUSED sums
+//                                           (without sums it does not have to wait either);
+//   U::coefficients(record, prep, log of this pass)            this pass's coefficients;
+//   U::fast_drift, U::fast_powers           both of the latter for alpha = 1, on two warps at once.
+// These are out of line and keep their state in shared memory: inlined, they cost the
+// marching loop 6 % (registers), and in local memory the update misses L1, which the
+// wait drops.  On return every thread may read the records.  False if a wait timed out.
+__device__ __forceinline__ double* pass_log(const PassArgs& P, int pass, int lat) {
+  return P.log && lat == 0 ? P.log + ADJ_LOG_W * (P.log_base + pass) : nullptr;
+}
+static __device__ __noinline__ void pass_weights_of(const PassStep* steps, PassStep one, int done, int next,
+                                                    TailPrep* q) {
+  const PassStep st = steps && done >= 0 ? steps[done] : one;
+  const PassStep nx = steps && next >= 0 ? steps[next] : one;
+  q->wout = st.wout;
+  q->win = st.win;
+  q->dnext = st.dnext;
+  q->ckn = nx.ck;
+  q->dnn = nx.dnext;
+}
+template <class Rec>
+static __device__ __noinline__ void load_run(const LatConst* L, const LatScalars* sc, Rec* r) {
+  r->L = *L;
+  load_state_cg(r->W, sc);
+}
+template <typename T, int NA, bool MOWN, int NUSED, class U>
+__device__ __forceinline__ bool ring_pass_begin(const Ring& R, const PassArgs& P, int pass, int ns, int ptot,
+                                                int parity, bool rev, int warp, int lane) {
+  typename U::Rec* const rec = reinterpret_cast<typename U::Rec*>(R.runs);
+  TailPrep* const prep = reinterpret_cast<TailPrep*>(R.runs + P.nrun_max * sizeof(typename U::Rec)) + lane;
+  const int nruns = R.flag[1];
+  const bool mine = warp == CONSUMER_WARPS - 1;
+  auto advance = [&](int r) {
+    const bool logs = blockIdx.x == 0;
+    if (pass > 0)
+      U::update(&rec[r], prep, R.red + lane * NQ, logs ? pass_log(P, pass - 1, prep->lat) : nullptr, nullptr, 0);
+    U::coefficients(&rec[r], prep, logs ? pass_log(P, pass, prep->lat) : nullptr);
+  };
+  auto ready = [&](int r) {
+    prep->lat = ring_run(R, ns, r).lat;
+    if (pass == 0) U::load(P, prep->lat, &rec[r]);
+    U::ready(P, pass - 1, pass, &rec[r], prep);
+    if (NUSED == 0) advance(r);
+  };
+  if (mine && lane < nruns) ready(lane);
+  if (pass > 0) {
+    if (threadIdx.x == 0 && !R.flag[0] && !wait_counter(P.gsync, gridDim.x * (unsigned)pass, P.wait_limit_ns))
+      R.flag[0] = 1;
+    __syncthreads();
+    if (R.flag[0]) return false;
   }
-  __syncthreads();
+  if (warp < R.S && warp < ptot) {
+    if (pass > 0) fence_proxy_async_global();
+    ring_issue_warp<T, NA, MOWN>(R, rev ? ptot - 1 - warp : warp, (pass * ptot + warp) % R.S, parity, lane);
+  }
+  for (int base = 0; base < nruns; base += 32) {
+    const int nb = min(32, nruns - base);
+    if (pass > 0 && NUSED > 0) {
+      ring_slot_sums<NUSED>(R, P, pass - 1, ns, nb, warp, lane, [&](int l) { return base + l; });
+      __syncthreads();
+    }
+    if (mine && lane < nb) {
+      if (base > 0) ready(base + lane);
+      if (pass > 0 && prep->fast) U::fast_drift(&rec[base + lane], prep, R.red + lane * NQ);
+      else if (NUSED > 0) advance(base + lane);
+    }
+    if (NUSED > 0 && pass > 0) {
+      if (base > 0) __syncthreads();  // prep is this round's
+      if (warp == CONSUMER_WARPS - 2 && lane < nb && prep->fast) {
+        const bool logs = blockIdx.x == 0;
+        U::fast_powers(&rec[base + lane], prep, R.red + lane * NQ, logs ? pass_log(P, pass - 1, prep->lat) : nullptr,
+                       logs ? pass_log(P, pass, prep->lat) : nullptr);
+      }
+    }
+    __syncthreads();
+  }
+  return true;
 }
 
-// Between two passes of one launch (warp 0, all lanes): the previous pass's
-// writes are all done before any of its planes is read; the first planes of
-// the pass are issued; then the updated scalars are awaited.
-template <typename T, int NA, bool MOWN = false>
-__device__ void ring_pass_start(const Ring& R, const PassArgs& P, int pass, int ptot, int parity, int lane) {
-  int go = 0;
-  if (lane == 0) {
-    if (pass > 0 && !R.flag[0] && !wait_counter(&P.gsync[0], gridDim.x * (unsigned)pass, P.wait_limit_ns))
-      R.flag[0] = 1;
-    go = !R.flag[0];
+// End of a pass (all threads): before another pass of the launch, the CTA's writes
+// are done and counted; after the last one, the lattices whose arrival count this CTA
+// completed are updated and U::store(P, lattice, record) leaves them in global memory.
+template <int NUSED, class U>
+__device__ __forceinline__ void ring_pass_end(const Ring& R, const PassArgs& P, int pass, int ns, int warp,
+                                              int lane) {
+  __syncthreads();
+  if (!last_pass(P, pass)) {
+    if (threadIdx.x == 0) {
+      fence_proxy_async_global();
+      red_release_inc(P.gsync);
+    }
+    return;
   }
-  go = __shfl_sync(0xffffffffu, go, 0);
-  if (pass > 0) fence_proxy_async_global();
-  if (go)
-    for (int g = 0; g < R.S && g < ptot; ++g)
-      ring_issue_warp<T, NA, MOWN>(R, g, (pass * ptot + g) % R.S, parity, lane);
-  if (lane == 0 && pass > 0 && !R.flag[0] &&
-      !wait_counter(&P.gsync[1], (unsigned)P.nlat * (unsigned)pass, P.wait_limit_ns))
-    R.flag[0] = 1;
+  typename U::Rec* const rec = reinterpret_cast<typename U::Rec*>(R.runs);
+  TailPrep* const prep = reinterpret_cast<TailPrep*>(R.runs + P.nrun_max * sizeof(typename U::Rec)) + lane;
+  const int npend = R.flag[3];
+  for (int base = 0; base < npend; base += 32) {
+    const int nb = min(32, npend - base);
+    __threadfence();
+    ring_slot_sums<NUSED>(R, P, pass, ns, nb, warp, lane, [&](int l) { return R.pend[base + l]; });
+    __syncthreads();
+    if (warp == CONSUMER_WARPS - 1 && lane < nb) {
+      const int r = R.pend[base + lane], lat = ring_run(R, ns, r).lat;
+      prep->lat = lat;
+      U::ready(P, pass, -1, &rec[r], prep);
+      if (prep->fast) {
+        U::fast_drift(&rec[r], prep, R.red + lane * NQ);
+        U::fast_powers(&rec[r], prep, R.red + lane * NQ, pass_log(P, pass, lat), nullptr);
+      } else {
+        U::update(&rec[r], prep, R.red + lane * NQ, pass_log(P, pass, lat), &P.sc[lat].obs, P.set_rho0);
+      }
+      U::store(P, lat, &rec[r]);
+      P.counters[lat] = 0u;
+    }
+    __syncthreads();
+  }
 }
 
 // After a timed-out wait (thread 0): wait, bounded, for copies still in

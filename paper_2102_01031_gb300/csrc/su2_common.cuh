@@ -213,7 +213,7 @@ __device__ void su2_pass_end(const PassArgs& P, const LatConst& L, Acc<T> (&acc)
     W.pi2 = spost;
     W.pi2A = slinks;
   }
-  advance_scalars(P, L, W, E, RED > 0);
+  advance_scalars(PassStep{P.ck, P.wout, P.win, P.dnext}, L, W, E, RED > 0);
   if (RED == 2) {
     cl_energies_t& ob = P.sc->obs;
     for (int k2 = 0; k2 < 4; ++k2) {
@@ -242,9 +242,9 @@ __device__ void su2_pass_end(const PassArgs& P, const LatConst& L, Acc<T> (&acc)
     ob.EKB = EKB;
     ob.EGB = EGB;
     ob.nonfinite = (int64_t)red_s[NACC][0];
-    finish_obs(P, L, W, ob);
+    finish_obs(P.set_rho0, L, W, ob);
   }
-  advance_drift(P, L, W);
+  advance_drift(P.dnext, L, W);
   store_state(P.sc, W);
   P.counters[0] = 0u;
   __threadfence();

@@ -1,6 +1,6 @@
-// tail.cuh -- per-lattice scalar update run by the last CTA of a DK pass:
-// Friedmann kicks of b = a', the next drift coefficient, and the packaging of
-// measured volume averages.  FP64 throughout.
+// tail.cuh -- the per-lattice scalar update between two DK passes: Friedmann
+// kicks of b = a', the next drift coefficient, and the packaging of measured
+// volume averages.  FP64 throughout.
 #pragma once
 
 #include <cstddef>
@@ -60,30 +60,30 @@ __device__ __forceinline__ double ipow(double x, int n) {
 
 // a^(m alpha + k): by multiplication when alpha is a small integer (alpha = 1
 // or 0 in the manual's scenarios), pow otherwise.
-__device__ __forceinline__ double apow(const LatConst& L, double a, int m, int k) {
+__device__ __forceinline__ double apow(const LatPar& L, double a, int m, int k) {
   if (L.int_alpha) return ipow(a, m * L.alpha_i + k);
   return pow_out_of_line(a, m * L.alpha + k);
 }
 
-__device__ __forceinline__ double fixed_p(const LatConst& L) {
+__device__ __forceinline__ double fixed_p(const LatPar& L) {
   return 2.0 / (3.0 * (1.0 + L.omega_eos) - 2.0 * L.alpha);
 }
 
 // Fixed power-law background, eq. ScaleFactorPowerLaw.
 template <class SS>
-__device__ __forceinline__ double a_fixed(const LatConst& L, const SS& S, double eta) {
+__device__ __forceinline__ double a_fixed(const LatPar& L, const SS& S, double eta) {
   double p = fixed_p(L);
   return S.a0 * pow_out_of_line(1.0 + S.Hfix * (eta - S.eta0) / p, p);
 }
 template <class SS>
-__device__ __forceinline__ double H_fixed(const LatConst& L, const SS& S, double eta) {
+__device__ __forceinline__ double H_fixed(const LatPar& L, const SS& S, double eta) {
   double p = fixed_p(L);
   return S.Hfix / (1.0 + S.Hfix * (eta - S.eta0) / p);
 }
 
 // b' = K_a (Sec. 3.5.2 / Sec. 4.3): a^{2alpha+1}/3 (f_s/m_p)^2 [(alpha-2) E_K + alpha E_G
 //        + (alpha-1)(E_K^A + E_G^A) + (alpha+1) E_V]
-__device__ __forceinline__ double kernel_a(const LatConst& L, double a, double EK, double EG,
+__device__ __forceinline__ double kernel_a(const LatPar& L, double a, double EK, double EG,
                                            double EV, double EKA, double EGA) {
   const double al = L.alpha;
   return apow(L, a, 2, 1) * (1.0 / 3.0) * L.fm2 *
@@ -91,7 +91,7 @@ __device__ __forceinline__ double kernel_a(const LatConst& L, double a, double E
 }
 
 // The factor a^{2alpha+1}/3 (f_s/m_p)^2 that both Friedmann kicks of a pass share.
-__device__ __forceinline__ double kernel_a_pref(const LatConst& L, double a) {
+__device__ __forceinline__ double kernel_a_pref(const LatPar& L, double a) {
   return apow(L, a, 2, 1) * (1.0 / 3.0) * L.fm2;
 }
 
@@ -99,7 +99,7 @@ __device__ __forceinline__ double kernel_a_pref(const LatConst& L, double a) {
 // the post-kick momenta, as in the velocity-Verlet step), pref = kernel_a_pref
 // at the current a.
 template <class SS>
-__device__ inline void advance_scalars(const PassArgs& P, const LatConst& L, SS& S,
+__device__ inline void advance_scalars(const PassStep& P, const LatPar& L, SS& S,
                                        const PassSums& E, bool have_sums, double pref) {
   if (have_sums && L.expansion == CL_EXP_SELF) {
     const double al = L.alpha;
@@ -109,20 +109,20 @@ __device__ inline void advance_scalars(const PassArgs& P, const LatConst& L, SS&
   }
 }
 template <class SS>
-__device__ inline void advance_scalars(const PassArgs& P, const LatConst& L, SS& S,
+__device__ inline void advance_scalars(const PassStep& P, const LatPar& L, SS& S,
                                        const PassSums& E, bool have_sums) {
   if (have_sums && L.expansion == CL_EXP_SELF) advance_scalars(P, L, S, E, true, kernel_a_pref(L, S.a));
 }
 
 // The two Friedmann kicks of a pass for the scalar models (no U(1) energies),
 // merged:  b += pref [(alpha-2)(w_out E_K^pre + w_in E_K^post) + (w_out + w_in)(alpha E_G + (alpha+1) E_V)].
-// FriedPre holds the factors that do not depend on the pass's sums.
+// FriedPre holds the factors that do not depend on the pass's sums (pref = kernel_a_pref at the current a).
 struct FriedPre {
   double pref, am2, al, ap1, wout, win, ws;
 };
-__device__ __forceinline__ FriedPre friedmann_pre(const LatConst& L, double a, double wout, double win) {
+__device__ __forceinline__ FriedPre friedmann_pre(const LatPar& L, double pref, double wout, double win) {
   FriedPre F;
-  F.pref = kernel_a_pref(L, a);
+  F.pref = pref;
   F.al = L.alpha;
   F.am2 = L.alpha - 2.0;
   F.ap1 = L.alpha + 1.0;
@@ -140,7 +140,7 @@ __device__ __forceinline__ double friedmann_kicks_scalar(const FriedPre& F, cons
 // w_in dK_a/da + w_out dK_a/da of the two Friedmann kicks of a pass (scalar
 // fields), at fixed fields and momenta: with E_K ~ a^-6, E_G ~ a^-2,
 //   d/da [a^{2alpha+1} E] = a^{2alpha} (2alpha+1-s) E  for E ~ a^-s.
-__device__ __forceinline__ double kernel_a_da(const PassArgs& P, const LatConst& L, double a,
+__device__ __forceinline__ double kernel_a_da(const PassStep& P, const LatPar& L, double a,
                                               const PassSums& E) {
   const double al = L.alpha, w = P.win + P.wout;
   return apow(L, a, 2, 0) * (1.0 / 3.0) * L.fm2 *
@@ -148,16 +148,16 @@ __device__ __forceinline__ double kernel_a_da(const PassArgs& P, const LatConst&
           w * ((2.0 * al - 1.0) * al * E.EG + (2.0 * al + 1.0) * (al + 1.0) * E.EV));
 }
 
-// The drift of a by P.dnext and the drift coefficients of the next pass:
-//   a' = a + dnext b (self-consistent) or a(eta + dnext) (fixed power law),
-//   cd = dnext abar^{alpha-3}, cdA = dnext abar^{alpha-1}, abar = (a + a')/2,
+// The drift of a by dn and the drift coefficients of the next pass:
+//   a' = a + dn b (self-consistent) or a(eta + dn) (fixed power law),
+//   cd = dn abar^{alpha-3}, cdA = dn abar^{alpha-1}, abar = (a + a')/2,
 //   and the kick's a'^{1+alpha}, a'^{3+alpha}, a'^{alpha-1}.
 // Few FP64 operations: alpha's exponents are read once, negative powers are
 // reciprocals of positive ones, and alpha = 1 (the manual's default) is
 // straight-line code.
 // Drift coefficients of a drift dn at the midpoint scale factor abar: fields
 // h abar^{alpha-3}, links h abar^{alpha-1} (Sec. 3.5.2; Sec. 4.3 for the links).
-__device__ inline void drift_coefficients(const LatConst& L, double abar, double dn, double& cd, double& cdA) {
+__device__ inline void drift_coefficients(const LatPar& L, double abar, double dn, double& cd, double& cdA) {
   const int ia = L.alpha_i;
   if (L.int_alpha && ia == 1) {
     cd = dn * (1.0 / (abar * abar));
@@ -172,8 +172,8 @@ __device__ inline void drift_coefficients(const LatConst& L, double abar, double
 }
 
 template <class SS>
-__device__ inline void advance_drift(const PassArgs& P, const LatConst& L, SS& S) {
-  const double a = S.a, dn = P.dnext;
+__device__ inline void advance_drift(double dn, const LatPar& L, SS& S) {
+  const double a = S.a;
   if (dn == 0.0) {
     S.cd = 0.0;
     S.cdA = 0.0;
@@ -205,9 +205,49 @@ __device__ inline void advance_drift(const PassArgs& P, const LatConst& L, SS& S
   }
 }
 
+// The same for alpha = 1 with self-consistent expansion.  Between two passes every
+// CTA waits for this, and on this part an FP64 operation takes about 100 cycles (64
+// even when it depends on nothing), so the work is cut to its dependent minimum:
+//   alpha1_ready, before the wait for the sums: with K_a = (a^3/3)(f_s/m_p)^2 [-E_K + E_G + 2 E_V],
+//     E_K = s_kin/(2 a^6 V), E_G = s_grad/(2 a^2 dx^2 V), E_V = s_pot/V, the kicked b as a
+//     linear form of the pass's sums (kin_pre: the pre-kick sum of pi^2);
+//   then on two warps at once alpha1_drift (the division) and alpha1_powers.
+// One thread doing all of it took 4400 cycles between the sums and the next pass.
+__device__ __forceinline__ void alpha1_ready(const LatPar& L, const ScalarState& W, TailPrep* q) {
+  const double K = L.fm2 * (1.0 / 6.0) * L.inv_V, ws = q->wout + q->win;
+  const double a = W.a, a3 = a * a * a, k3 = K / a3;
+  q->fast = 1;
+  q->a = a;
+  q->pi2 = W.pi2;
+  q->b0 = fma(-q->wout * k3, W.pi2, W.b);
+  q->c[0] = -q->win * k3;
+  q->c[1] = ws * (K * L.inv_dx2) * a;
+  q->c[2] = 4.0 * ws * K * a3;
+}
+__device__ __forceinline__ double alpha1_b(const TailPrep* q, double kin, double grad, double pot) {
+  return fma(q->c[0], kin, fma(q->c[1], grad, fma(q->c[2], pot, q->b0)));
+}
+// b and the drift coefficients at the midpoint scale factor
+__device__ __forceinline__ void alpha1_drift(ScalarState& W, const TailPrep* q, double b) {
+  const double dn = q->dnext, abar = fma(0.5 * dn, b, q->a);
+  W.b = b;
+  W.cd = dn == 0.0 ? 0.0 : dn / (abar * abar);
+  W.cdA = dn;
+  W.eta += dn;
+}
+// a and its powers after the drift
+__device__ __forceinline__ void alpha1_powers(ScalarState& W, const TailPrep* q, double b) {
+  const double an = fma(q->dnext, b, q->a), an2 = an * an;
+  W.a = an;
+  if (q->dnext == 0.0) return;
+  W.apow1 = an2;
+  W.apow3 = an2 * an2;
+  W.apowm1 = 1.0;
+}
+
 // Hubble-constraint monitor and energy bookkeeping of a measurement.
 template <class SS>
-__device__ inline void finish_obs(const PassArgs& P, const LatConst& L, SS& S, cl_energies_t& o) {
+__device__ inline void finish_obs(int set_rho0, const LatPar& L, SS& S, cl_energies_t& o) {
   double rho = o.EKA + o.EGA + o.EKB + o.EGB;
   for (int k = 0; k < 4; ++k) rho += o.EK[k] + o.EG[k] + o.EV[k];
   o.rho = rho;
@@ -215,7 +255,7 @@ __device__ inline void finish_obs(const PassArgs& P, const LatConst& L, SS& S, c
   o.hubble_rhs = apow(L, S.a, 2, 2) * (1.0 / 3.0) * L.fm2 * rho;
   const double den = o.hubble_lhs + o.hubble_rhs;
   o.hubble_viol = den > 0.0 ? (o.hubble_lhs - o.hubble_rhs) / den : 0.0;
-  if (P.set_rho0) S.rho0 = rho;
+  if (set_rho0) S.rho0 = rho;
   o.energy_cons = S.rho0 != 0.0 ? 1.0 - rho / S.rho0 : 0.0;
   o.eta = S.eta;
   o.a = S.a;
