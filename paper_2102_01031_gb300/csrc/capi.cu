@@ -52,13 +52,13 @@ cudaError_t launch_ic_modes(double2*, double2*, const LatConst*, const LatScalar
 cudaError_t launch_ic_assemble(int, void*, void*, const double2*, const double2*, const LatConst*,
                                const LatScalars*, double, double, long long, cudaStream_t);
 cudaError_t launch_fft_axis(double2*, const FftPlan&, cudaStream_t);
-cudaError_t launch_fft_twiddles(double2*, int, cudaStream_t);
+cudaError_t launch_fft_twiddles(int4*, int, int, cudaStream_t);
 cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftPlan& pl, double dk, int nb,
                                  int nblk, double* part, double kIR, double dx, double* out, cudaStream_t st,
                                  const int* bin_of, const double* geo);
 cudaError_t launch_shell_geometry(int N, double dk, int nb, int nblk, int* bin_of, double* geo, double* part,
                                   cudaStream_t st);
-int fft_batch(int N);
+FftPlan fft_plan(int N, int sign, const int4* tw, int pitch, int nu);
 cudaError_t launch_to_complex(int, const void*, double2*, long long, cudaStream_t);
 cudaError_t launch_bins(const double2*, int, double, int, int, double*, double, double, double*,
                         cudaStream_t, int raw = 0);
@@ -154,7 +154,7 @@ struct cl_ctx {
   unsigned* d_cnt = nullptr;       // [nlat]
   double* d_tmp = nullptr;         // scratch for conversions / monitors (vmax doubles)
   double2* d_cplx = nullptr;       // scratch complex (2 vmax)
-  double2* d_tw = nullptr;         // FFT twiddle table (the largest lattice's N entries)
+  int4* d_tw = nullptr;         // FFT twiddle table (the largest lattice's N entries)
   double* d_spec = nullptr;        // spectrum scratch: block rows (3 x 2048 x nblk), per-lattice bins, mean
   int spec_lats = 0;               // lattices d_spec has room for
   int* d_bin_of = nullptr;         // cached shell geometry of (geo_N, geo_dk): bin of each |n|^2,
@@ -269,14 +269,6 @@ void append_pass_steps(int integrator, double h, int n, bool& open, double& dpre
 // The pass that closes a stream: the kick-out of the last drift, no drift.
 PassStep closing_pass_step(double dprev) { return PassStep{0.5 * dprev, 0.5 * dprev, 0.0, 0.0}; }
 
-void fft_radices(int N, FftPlan& pl) {
-  pl.nrad = 0;
-  int m = N;
-  while (m % 4 == 0) { pl.rad[pl.nrad++] = 4; m /= 4; }
-  while (m % 2 == 0) { pl.rad[pl.nrad++] = 2; m /= 2; }
-  while (m % 3 == 0) { pl.rad[pl.nrad++] = 3; m /= 3; }
-}
-
 void* arr_ptr(cl_ctx* c, int lat, int parity, int a) {
   const LatHost& L = c->lats[lat];
   if (L.bound[0]) return (char*)L.bound[parity] + (size_t)a * L.V * c->esz;
@@ -284,14 +276,8 @@ void* arr_ptr(cl_ctx* c, int lat, int parity, int a) {
 }
 
 cl_status fft3d(cl_ctx* c, int N, double2* data, int sign) {
-  FftPlan pl;
-  pl.N = N;
-  pl.sign = sign;
-  pl.batch = fft_batch(N);
-  pl.tw = c->d_tw;
-  pl.pitch = pl.nu = N;
-  fft_radices(N, pl);
-  CU(launch_fft_twiddles(c->d_tw, N, c->stream));
+  FftPlan pl = fft_plan(N, sign, c->d_tw, N, N);
+  CU(launch_fft_twiddles(c->d_tw, N, sign, c->stream));
   ++c->launches;
   for (int axis = 0; axis < 3; ++axis) {
     pl.axis = axis;
@@ -1041,7 +1027,7 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
   CU(cudaMemcpyAsync(c->d_cta, cta.data(), cta.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   // initial conditions, lattice by lattice
   CU(cudaMalloc(&c->d_cplx, 2 * (size_t)c->vmax * sizeof(double2)));
-  CU(cudaMalloc(&c->d_tw, 512 * sizeof(double2)));
+  CU(cudaMalloc(&c->d_tw, 512 * sizeof(int4)));
   CU(cudaMalloc(&c->d_tmp, std::max<size_t>((size_t)c->vmax, 1 << 16) * sizeof(double)));
   for (int l = 0; l < c->nlat; ++l) {
     const LatHost& H = c->lats[l];
@@ -1231,7 +1217,7 @@ static cl_status su2_init(cl_ctx* c, int N, double kIR, uint64_t seed) {
     for (int a = 0; a < MAX_ARR; ++a) L.buf[par][a] = arr_ptr(c, 0, par, a);
   CU(cudaMemcpyAsync(c->d_lat, &L, sizeof(LatConst), cudaMemcpyHostToDevice, c->stream));
   CU(cudaMalloc(&c->d_cplx, 2 * (size_t)H.V * sizeof(double2)));
-  CU(cudaMalloc(&c->d_tw, 512 * sizeof(double2)));
+  CU(cudaMalloc(&c->d_tw, 512 * sizeof(int4)));
   CU(cudaMalloc(&c->d_tmp, std::max<size_t>((size_t)H.V, 1 << 16) * sizeof(double)));
   ICArgs A;
   memset(&A, 0, sizeof(A));
@@ -1540,15 +1526,8 @@ cl_status cl_ensemble_spectrum(cl_ctx* c, const int* lats, int nl, int field, in
   double* mean = bins + (size_t)nl * 3 * nb;
   double2* F = c->d_cplx;
   // real fields: the half spectrum (row pairs along x, then the N/2 + 1 columns kept along y and z)
-  FftPlan pl;
-  pl.N = H.N;
-  pl.sign = -1;
-  pl.batch = fft_batch(H.N);
-  pl.tw = c->d_tw;
-  pl.pitch = pl.nu = H.N;
-  pl.axis = 0;
-  fft_radices(H.N, pl);
-  CU(launch_fft_twiddles(c->d_tw, H.N, c->stream));
+  const FftPlan pl = fft_plan(H.N, -1, c->d_tw, H.N, H.N);
+  CU(launch_fft_twiddles(c->d_tw, H.N, pl.sign, c->stream));
   ++c->launches;
   if (c->geo_N != H.N || c->geo_dk != dk_bin) {  // the shells of (N, dk_bin), kept for later calls
     CU(cudaStreamSynchronize(c->stream));

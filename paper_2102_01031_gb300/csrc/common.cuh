@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fix_fft.h"   // FastDiv
 #include "worklist.h"  // Seg, MAX_SEG_PER_CTA
 
 #include "cl.h"
@@ -184,14 +185,22 @@ struct ICArgs {
   int model, nf;
 };
 
-// One batched 1-D FFT along `axis` of an N^3 complex array.
+// One batched 1-D FFT along `axis` of an N^3 complex array (fft_plan in ic_fft.cu fills
+// in everything but axis; a division by a runtime number costs a thread more than a
+// butterfly's sums, so every divisor comes with its multiplier).
+struct FftStage {
+  int R, Ns, ts;         // radix, sub-length before it, table stride of its roots
+  FastDiv NR, dNs;       // N / R, Ns
+};
 struct FftPlan {
   int N, nrad, axis, sign;
-  int rad[16];
+  FftStage st[8];
   int batch;             // lines per CTA (a divisor of N)
-  const double2* tw;     // tw[e] = exp(+2 pi i e/N), e < N
+  const int4* tw;        // exp(sign 2 pi i e/N), e < N, in fixed point (fft_twiddle_kernel)
   int pitch;             // x extent of the array in memory (N; N/2 + 1 for a half spectrum)
   int nu;                // lines along the fastest other index (axes 1, 2: the columns kept, <= pitch)
+  int ng;                // groups of `batch` lines among them
+  FastDiv dN, dB, dH, dg;  // N, batch, N/2 + 1, ng
 };
 
 // ---------------------------------------------------------------------------

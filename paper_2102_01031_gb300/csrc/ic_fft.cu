@@ -10,9 +10,13 @@
 // keyed by the seed, with counter (Fourier index, field, draw, 0).  Only the
 // member of each (n, -n) pair with the smaller index is drawn; its partner is
 // the complex conjugate so that the field is real.
+#include <limits.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "common.cuh"
+#include "fix_fft.h"
 
 namespace clg {
 
@@ -271,122 +275,245 @@ template __global__ void ic_assemble_kernel<double>(double*, double*, const doub
 //   y[(j/Ns) Ns R + k + q Ns] = sum_r v_r exp(sign 2 pi i r q / R).
 // The twiddles come from a table of the N-th roots of unity (w^{k r} is root
 // (k r mod Ns R) N/(Ns R)), made once per transform by fft_twiddle_kernel.
+//
+// The arithmetic is 64-bit fixed point with one exponent per line (fix_fft.h).
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
-}
-
-__global__ void fft_twiddle_kernel(double2* tw, int N) {
+__global__ void fft_twiddle_kernel(int4* tw, int N, int sign) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N) return;
   double sn, cs;
   sincospi(2.0 * (double)e / (double)N, &sn, &cs);
-  tw[e] = make_double2(cs, sn);
+  int ch, cl, sh, sl;
+  root_words(cs, ch, cl);
+  root_words(sign * sn, sh, sl);
+  tw[e] = make_int4(ch, cl, sh, sl);
+}
+__device__ __forceinline__ CFix cmul(const CFix& a, const int4& w) { return cmul(a, w.x, w.y, w.z, w.w); }
+
+// One Stockham stage of radix R from a into b (B lines of pitch Pt).
+template <int R>
+__device__ __forceinline__ void stockham_stage(const CFix* a, CFix* b, const int4* w, const FftStage& st, int sign,
+                                               int B, int Pt) {
+  const int NR = (int)st.NR.d, Ns = st.Ns, ts = st.ts;
+  for (int t = threadIdx.x; t < B * NR; t += blockDim.x) {
+    const int line = st.NR.div(t), j = st.NR.mod(t, line);
+    const int g = st.dNs.div(j), k = st.dNs.mod(j, g);
+    const CFix* ai = a + line * Pt + j;
+    CFix v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ai[r * NR];
+    if (Ns > 1) {
+      const int4* wk = w + k * ts;  // k r < Ns R, so no reduction
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], wk[(r - 1) * k * ts]);
+    }
+    butterfly<R>(v, sign);
+    CFix* bo = b + line * Pt + g * (Ns * R) + k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) bo[q * Ns] = v[q];
+  }
+}
+
+// The same with the line length N, the batch B and the sub-length Ns compiled in: for the
+// sizes runs are made at (128, 256, 512), where the index arithmetic of runtime sizes was a
+// fifth of the instructions (256^3: 223 -> 185 us for the row pairs, 194 -> 166 us an axis).
+template <int N, int B, int R, int Ns>
+__device__ __forceinline__ void stockham_stage_of(const CFix* a, CFix* b, const int4* w, int sign) {
+  constexpr int NR = N / R, ts = N / (Ns * R), Pt = N + 1;
+#pragma unroll 1
+  for (int t = threadIdx.x; t < B * NR; t += blockDim.x) {
+    const int line = t / NR, j = t % NR, g = j / Ns, k = j % Ns;
+    const CFix* ai = a + line * Pt + j;
+    CFix v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ai[r * NR];
+    if (Ns > 1) {
+      const int4* wk = w + k * ts;
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], wk[(r - 1) * k * ts]);
+    }
+    butterfly<R>(v, sign);
+    CFix* bo = b + line * Pt + g * (Ns * R) + k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) bo[q * Ns] = v[q];
+  }
+}
+template <int N, int B, int Ns = 1>
+__device__ __forceinline__ CFix* stockham_lines_of(CFix* a, CFix* b, const int4* w, int sign) {
+  if constexpr (Ns == N) {
+    return a;
+  } else {
+    constexpr int m = N / Ns, R = m % 4 == 0 ? 4 : (m % 2 == 0 ? 2 : 3);
+    stockham_stage_of<N, B, R, Ns>(a, b, w, sign);
+    __syncthreads();
+    return stockham_lines_of<N, B, Ns * R>(b, a, w, sign);
+  }
 }
 
 // The Stockham stages on B lines held in shared memory (line pitch Pt), the
 // roots of unity in w; returns the buffer (a or b) that holds the result.
-__device__ double2* stockham_lines(double2* a, double2* b, const double2* w, const FftPlan& plan, int B, int Pt) {
-  const int N = plan.N, nt = blockDim.x, tid = threadIdx.x;
-  int Ns = 1;
+__device__ __forceinline__ CFix* stockham_lines(CFix* a, CFix* b, const int4* w, const FftPlan& plan, int B, int Pt) {
   for (int s = 0; s < plan.nrad; ++s) {
-    const int R = plan.rad[s];
-    const int NR = N / R;
-    const int L = Ns * R;
-    const int ts = N / L;  // table stride of this stage's roots
-    for (int t = tid; t < B * NR; t += nt) {
-      const int j = t % NR, line = t / NR;
-      const double2* ai = a + line * Pt;
-      const int k = j % Ns;
-      double2 v[4];
-      for (int r = 0; r < R; ++r) {
-        double2 x = ai[j + r * NR];
-        if (k != 0 && r != 0) x = cmul(x, w[((k * r) % L) * ts]);
-        v[r] = x;
-      }
-      double2 o[4];
-      if (R == 2) {
-        o[0] = make_double2(v[0].x + v[1].x, v[0].y + v[1].y);
-        o[1] = make_double2(v[0].x - v[1].x, v[0].y - v[1].y);
-      } else if (R == 4) {
-        // j = sign * i
-        const double2 t0 = make_double2(v[0].x + v[2].x, v[0].y + v[2].y);
-        const double2 t1 = make_double2(v[0].x - v[2].x, v[0].y - v[2].y);
-        const double2 t2 = make_double2(v[1].x + v[3].x, v[1].y + v[3].y);
-        const double2 d = make_double2(v[1].x - v[3].x, v[1].y - v[3].y);
-        const double2 t3 = make_double2(-plan.sign * d.y, plan.sign * d.x);  // j*(v1 - v3)
-        o[0] = make_double2(t0.x + t2.x, t0.y + t2.y);
-        o[1] = make_double2(t1.x + t3.x, t1.y + t3.y);
-        o[2] = make_double2(t0.x - t2.x, t0.y - t2.y);
-        o[3] = make_double2(t1.x - t3.x, t1.y - t3.y);
-      } else {  // R == 3, w = (-1/2, sign sqrt3/2)
-        const double h = 0.86602540378443864676 * plan.sign;
-        const double2 s3 = make_double2(v[1].x + v[2].x, v[1].y + v[2].y);
-        const double2 d = make_double2(v[1].x - v[2].x, v[1].y - v[2].y);
-        const double2 m = make_double2(v[0].x - 0.5 * s3.x, v[0].y - 0.5 * s3.y);
-        o[0] = make_double2(v[0].x + s3.x, v[0].y + s3.y);
-        o[1] = make_double2(m.x - h * d.y, m.y + h * d.x);
-        o[2] = make_double2(m.x + h * d.y, m.y - h * d.x);
-      }
-      double2* bo = b + line * Pt + (j / Ns) * L + k;
-      for (int q2 = 0; q2 < R; ++q2) bo[q2 * Ns] = o[q2];
-    }
+    const FftStage& st = plan.st[s];
+    if (st.R == 4) stockham_stage<4>(a, b, w, st, plan.sign, B, Pt);
+    else if (st.R == 2) stockham_stage<2>(a, b, w, st, plan.sign, B, Pt);
+    else stockham_stage<3>(a, b, w, st, plan.sign, B, Pt);
     __syncthreads();
-    double2* t = a;
+    CFix* t = a;
     a = b;
     b = t;
-    Ns = L;
   }
   return a;
 }
 
-__device__ __forceinline__ void load_roots(double2* w, const FftPlan& plan) {
-  for (int e = threadIdx.x; e < plan.N; e += blockDim.x) {
-    const double2 t = plan.tw[e];
-    w[e] = make_double2(t.x, plan.sign * t.y);
+// A CTA's shared memory: two buffers of B lines, the roots, each line's largest high
+// word, sum of sizes and scale.
+struct FftSmem {
+  CFix *a, *b;
+  int4* w;
+  int *top, *sum;
+  LineScale* sc;
+};
+__device__ __forceinline__ FftSmem fft_smem(unsigned char* base, int N, int B) {
+  const int Pt = N + 1;  // padded line pitch: no bank conflicts across lines
+  FftSmem M;
+  M.a = reinterpret_cast<CFix*>(base);
+  M.b = M.a + B * Pt;
+  M.w = reinterpret_cast<int4*>(M.b + B * Pt);
+  M.top = reinterpret_cast<int*>(M.w + N);
+  M.sum = M.top + B;
+  M.sc = reinterpret_cast<LineScale*>(M.sum + B);
+  return M;
+}
+__device__ __forceinline__ void fft_begin(const FftSmem& M, const FftPlan& plan) {
+  for (int e = threadIdx.x; e < plan.N; e += blockDim.x) M.w[e] = plan.tw[e];
+  for (int l = threadIdx.x; l < plan.batch; l += blockDim.x) {
+    M.top[l] = 0;
+    M.sum[l] = 0;
+  }
+  __syncthreads();
+}
+// The largest (the sum) of v over a line into at[l]; all lanes of a warp call, those
+// with l < 0 contribute nothing.  A warp on one line adds up first: 32 updates of one
+// word take their turns.
+template <bool MAX>
+__device__ __forceinline__ void line_reduce(int* at, int l, int v) {
+  const int l0 = __shfl_sync(0xffffffffu, l, 0);
+  if (__all_sync(0xffffffffu, l == l0)) {
+    if (l0 < 0) return;
+    const int r = MAX ? __reduce_max_sync(0xffffffffu, v) : __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) {
+      if (MAX) atomicMax(&at[l0], r);
+      else atomicAdd(&at[l0], r);
+    }
+  } else if (l >= 0) {
+    if (MAX) atomicMax(&at[l], v);
+    else atomicAdd(&at[l], v);
   }
 }
+// Lines per CTA: the largest divisor of N with batch * N <= 2048 (at most 72 KB
+// of shared memory per CTA).
+__host__ __device__ constexpr int fft_batch_of(int N) {
+  int b = 1;
+  for (int d = 1; d <= N && d * N <= 2048; ++d)
+    if (N % d == 0) b = d;
+  return b;
+}
+constexpr int FFT_HELD = 4;  // elements a thread holds between its load and the line's exponent
 
 // Element (line u, position j) of an array of x extent P = plan.pitch:
 // axis 0: j + P (u + N w) (rows, P = N); axis 1: u + P (j + N w); axis 2: u + P (w + N j).
 // A CTA takes `batch` lines with consecutive u (and one w); lines with u >= nu are
 // not loaded or stored (the last group of a half spectrum's N/2 + 1 columns).
-__global__ void fft_lines_kernel(double2* data, const FftPlan plan) {
-  extern __shared__ double2 fbuf[];
-  const int N = plan.N, B = plan.batch, Pt = N + 1;  // padded line pitch: no bank conflicts across lines
+template <int NC>
+__global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const __grid_constant__ FftPlan plan) {
+  extern __shared__ __align__(16) unsigned char fbuf[];
+  const int N = NC ? NC : plan.N, B = NC ? fft_batch_of(NC) : plan.batch, Pt = N + 1;
   const int nt = blockDim.x, tid = threadIdx.x;
-  double2* a = fbuf;
-  double2* b = fbuf + B * Pt;
-  double2* w = fbuf + 2 * B * Pt;
+  const FftSmem M = fft_smem(fbuf, N, B);
   const int P = plan.pitch, nu = plan.nu;
-  const int ng = (nu + B - 1) / B;
-  const long long u0 = (long long)(blockIdx.x % ng) * B, ww = blockIdx.x / ng;
+  const int w0 = plan.dg.div(blockIdx.x);
+  const long long u0 = (long long)plan.dg.mod(blockIdx.x, w0) * B, ww = w0;
   const long long PN = (long long)P * N;
-  load_roots(w, plan);
-  if (plan.axis == 0) {
-    const double2* src = data + PN * ww + (long long)N * u0;  // B whole rows, contiguous
-    for (int t = tid; t < B * N; t += nt) a[(t / N) * Pt + t % N] = src[t];
+  fft_begin(M, plan);
+  // element t of the CTA: line l, position p, and its place in memory
+  const bool rows = plan.axis == 0;  // B whole rows, contiguous
+  const long long base = rows ? PN * ww + (long long)N * u0 : (plan.axis == 1 ? PN * ww + u0 : (long long)P * ww + u0);
+  const long long js = rows ? 0 : (plan.axis == 1 ? P : PN);
+  auto place = [&](int t, int& l, int& p) -> long long {
+    if (rows) {
+      l = NC ? t / N : plan.dN.div(t);
+      p = t - l * N;
+      return base + t;
+    }
+    p = NC ? t / B : plan.dB.div(t);
+    l = t - p * B;
+    return u0 + l < nu ? base + p * js + l : -1;
+  };
+  // load (the host picks nt so that a thread holds at most FFT_HELD elements), the
+  // lines' exponents and sums, fixed point
+  double2 h[FFT_HELD];
+  int hl[FFT_HELD];  // line; -1: nothing
+#pragma unroll
+  for (int i = 0; i < FFT_HELD; ++i) {
+    const int t = tid + i * nt;
+    int l = 0, p = 0;
+    const long long at = t < B * N ? place(t, l, p) : -1;
+    h[i] = at >= 0 ? data[at] : make_double2(0.0, 0.0);
+    hl[i] = at >= 0 ? l : -1;
+  }
+  // a thread's elements all lie on its first one's line where the block is a multiple of
+  // the batch (columns): one update of the line's words instead of FFT_HELD
+  const bool one = !rows && plan.dB.mod(nt, plan.dB.div(nt)) == 0;
+  int top[FFT_HELD];
+#pragma unroll
+  for (int i = 0; i < FFT_HELD; ++i) top[i] = max(top_of(h[i].x), top_of(h[i].y));
+  if (one) {
+    line_reduce<true>(M.top, hl[0], max(max(top[0], top[1]), max(top[2], top[3])));
   } else {
-    const long long base = plan.axis == 1 ? PN * ww + u0 : (long long)P * ww + u0;
-    const long long js = plan.axis == 1 ? P : PN;
-    for (int t = tid; t < B * N; t += nt) {
-      const int l = t % B;
-      a[l * Pt + t / B] = u0 + l < nu ? data[base + (t / B) * js + l] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int i = 0; i < FFT_HELD; ++i) line_reduce<true>(M.top, hl[i], top[i]);
+  }
+  __syncthreads();
+  int sum[FFT_HELD];
+#pragma unroll
+  for (int i = 0; i < FFT_HELD; ++i) {
+    const int E = expo_of<double>(hl[i] >= 0 ? M.top[hl[i]] : 0);
+    sum[i] = hl[i] >= 0 ? size_of(h[i].x, E) + size_of(h[i].y, E) : 0;
+  }
+  if (one) {
+    line_reduce<false>(M.sum, hl[0], (sum[0] + sum[1]) + (sum[2] + sum[3]));
+  } else {
+#pragma unroll
+    for (int i = 0; i < FFT_HELD; ++i) line_reduce<false>(M.sum, hl[i], sum[i]);
+  }
+  __syncthreads();
+  for (int l = tid; l < B; l += nt) M.sc[l] = line_scale<double>(expo_of<double>(M.top[l]), M.sum[l]);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < FFT_HELD; ++i) {
+    const int t = tid + i * nt;
+    if (t < B * N) {
+      int l = 0, p = 0;
+      place(t, l, p);
+      const LineScale sc = M.sc[l];
+      M.a[l * Pt + p] = CFix{to_fix(h[i].x, sc), to_fix(h[i].y, sc)};
     }
   }
   __syncthreads();
-  a = stockham_lines(a, b, w, plan, B, Pt);
-  if (plan.axis == 0) {
-    double2* dst = data + PN * ww + (long long)N * u0;
-    for (int t = tid; t < B * N; t += nt) dst[t] = a[(t / N) * Pt + t % N];
-  } else {
-    const long long base = plan.axis == 1 ? PN * ww + u0 : (long long)P * ww + u0;
-    const long long js = plan.axis == 1 ? P : PN;
-    for (int t = tid; t < B * N; t += nt) {
-      const int l = t % B;
-      if (u0 + l < nu) data[base + (t / B) * js + l] = a[l * Pt + t / B];
-    }
+  const CFix* a;
+  if constexpr (NC > 0) a = stockham_lines_of<NC, fft_batch_of(NC)>(M.a, M.b, M.w, plan.sign);
+  else a = stockham_lines(M.a, M.b, M.w, plan, B, Pt);
+  for (int t = tid; t < B * N; t += nt) {
+    int l = 0, p = 0;
+    const long long at = place(t, l, p);
+    if (at < 0) continue;
+    const LineScale sc = M.sc[l];
+    const int q = sc.E - FixIO<double>::BIAS - sc.up;
+    const CFix v = a[l * Pt + p];
+    data[at] = sc.E == FixIO<double>::ETOP
+                   ? make_double2(fix_nan(), fix_nan())
+                   : make_double2(from_fix(v.x, q, sc.plain), from_fix(v.y, q, sc.plain));
   }
 }
 
@@ -396,29 +523,58 @@ __global__ void fft_lines_kernel(double2* data, const FftPlan plan) {
 // row f_2p + i f_2p+1, Z = X_a + i X_b, and separated by the Hermitian symmetry
 // of real transforms: X_a(k) = (Z(k) + Z^*(N-k))/2, X_b(k) = (Z(k) - Z^*(N-k))/(2i),
 // for k = 0 .. N/2.  A CTA takes `batch` row pairs.
-template <typename T>
-__global__ void rfft_rows_kernel(const T* f, double2* H, const FftPlan plan) {
-  extern __shared__ double2 fbuf[];
-  const int N = plan.N, B = plan.batch, Pt = N + 1, NH = N / 2 + 1;
+template <typename T, int NC>
+__global__ void __launch_bounds__(512, 2) rfft_rows_kernel(const T* f, double2* H, const __grid_constant__ FftPlan plan) {
+  extern __shared__ __align__(16) unsigned char fbuf[];
+  const int N = NC ? NC : plan.N, B = NC ? fft_batch_of(NC) : plan.batch, Pt = N + 1, NH = N / 2 + 1;
   const int nt = blockDim.x, tid = threadIdx.x;
-  double2* a = fbuf;
-  double2* b = fbuf + B * Pt;
-  double2* w = fbuf + 2 * B * Pt;
+  const FftSmem M = fft_smem(fbuf, N, B);
   const long long p0 = (long long)blockIdx.x * B;  // first row pair of the CTA
-  load_roots(w, plan);
+  fft_begin(M, plan);
   const T* src = f + 2 * p0 * N;  // 2B whole rows, contiguous
-  for (int t = tid; t < 2 * B * N; t += nt) {
-    const int row = t / N, j = t % N;
-    double* slot = reinterpret_cast<double*>(&a[(row >> 1) * Pt + j]);
-    slot[row & 1] = (double)src[t];
+  auto row_of = [&](int t) { return NC ? t / N : plan.dN.div(t); };
+  T h[2 * FFT_HELD];
+#pragma unroll
+  for (int i = 0; i < 2 * FFT_HELD; ++i) {
+    const int t = tid + i * nt;
+    h[i] = t < 2 * B * N ? src[t] : T(0);
+  }
+#pragma unroll
+  for (int i = 0; i < 2 * FFT_HELD; ++i) {
+    const int t = tid + i * nt;
+    line_reduce<true>(M.top, t < 2 * B * N ? row_of(t) >> 1 : -1, top_of(h[i]));
   }
   __syncthreads();
-  a = stockham_lines(a, b, w, plan, B, Pt);
+#pragma unroll
+  for (int i = 0; i < 2 * FFT_HELD; ++i) {
+    const int t = tid + i * nt, l = t < 2 * B * N ? row_of(t) >> 1 : -1;
+    line_reduce<false>(M.sum, l, size_of(h[i], expo_of<T>(l >= 0 ? M.top[l] : 0)));
+  }
+  __syncthreads();
+  for (int l = tid; l < B; l += nt) M.sc[l] = line_scale<T>(expo_of<T>(M.top[l]), M.sum[l]);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 2 * FFT_HELD; ++i) {
+    const int t = tid + i * nt;
+    if (t < 2 * B * N) {
+      const int row = row_of(t), j = t - row * N;
+      fix* slot = reinterpret_cast<fix*>(&M.a[(row >> 1) * Pt + j]);
+      slot[row & 1] = to_fix(h[i], M.sc[row >> 1]);
+    }
+  }
+  __syncthreads();
+  const CFix* a;
+  if constexpr (NC > 0) a = stockham_lines_of<NC, fft_batch_of(NC)>(M.a, M.b, M.w, plan.sign);
+  else a = stockham_lines(M.a, M.b, M.w, plan, B, Pt);
   for (int t = tid; t < B * NH; t += nt) {
-    const int l = t / NH, k = t % NH;
-    const double2 Z = a[l * Pt + k], Y = a[l * Pt + (k == 0 ? 0 : N - k)];  // Y = Z(N - k)
-    const double2 Xa = make_double2(0.5 * (Z.x + Y.x), 0.5 * (Z.y - Y.y));
-    const double2 Xb = make_double2(0.5 * (Z.y + Y.y), 0.5 * (Y.x - Z.x));
+    const int l = NC ? t / NH : plan.dH.div(t), k = t - l * NH;
+    const CFix Z = a[l * Pt + k], Y = a[l * Pt + (k == 0 ? 0 : N - k)];  // Y = Z(N - k)
+    const LineScale sc = M.sc[l];
+    const int q = sc.E - FixIO<T>::BIAS - sc.up - 1;  // with the halves
+    // the sums are twice a row's transform, below 2^63
+    double2 Xa = make_double2(from_fix(Z.x + Y.x, q, sc.plain), from_fix(Z.y - Y.y, q, sc.plain));
+    double2 Xb = make_double2(from_fix(Z.y + Y.y, q, sc.plain), from_fix(Y.x - Z.x, q, sc.plain));
+    if (sc.E == FixIO<T>::ETOP) Xa.x = Xa.y = Xb.x = Xb.y = fix_nan();
     const long long ra = 2 * (p0 + l);
     H[ra * NH + k] = Xa;
     H[(ra + 1) * NH + k] = Xb;
@@ -628,31 +784,53 @@ __global__ void geo_partial_kernel(const int* bin_of, int N, int nb, double* par
   double* sc = sb + nb;
   for (int i = threadIdx.x; i < 2 * nb; i += blockDim.x) sb[i] = 0.0;
   __syncthreads();
-  const long long NN = (long long)N * N;
-  for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < NN; r += (long long)gridDim.x * blockDim.x) {
-    const int y = (int)(r % N), z = (int)(r / N);
-    const int ny = y <= N / 2 ? y : y - N, nz = z <= N / 2 ? z : z - N;
-    for (int x = 0; x < N; ++x) {  // one whole row per thread (this runs once per lattice size and bin width)
-      const int nx = x <= N / 2 ? x : x - N;
-      const int m2 = nx * nx + ny * ny + nz * nz;
-      const int b = bin_of[m2];
+  // one octant of the modes, |n_i| = 0 .. N/2, each standing for its mirror images
+  // (two per direction but for 0 and N/2): all of the N^3 modes one by one took 1.17 ms at 256^3
+  const int NH = N / 2 + 1;
+  auto images = [&](int n) { return n == 0 || n == N / 2 ? 1 : 2; };
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < NH * NH; r += gridDim.x * blockDim.x) {
+    const int ny = r % NH, nz = r / NH, wyz = images(ny) * images(nz);
+    int cur = -1;
+    double rn = 0.0, rc = 0.0;
+    for (int nx = 0; nx < NH; ++nx) {
+      const int m2 = nx * nx + ny * ny + nz * nz, b = bin_of[m2];
       if (b < 0) continue;
-      atomicAdd(&sn[b], sqrt((double)m2));
-      atomicAdd(&sc[b], 1.0);
+      if (b != cur) {
+        if (cur >= 0) {
+          atomicAdd(&sn[cur], rn);
+          atomicAdd(&sc[cur], rc);
+        }
+        cur = b;
+        rn = rc = 0.0;
+      }
+      const double w = (double)(wyz * images(nx));
+      rn = fma(w, sqrt((double)m2), rn);
+      rc += w;
+    }
+    if (cur >= 0) {
+      atomicAdd(&sn[cur], rn);
+      atomicAdd(&sc[cur], rc);
     }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < 2 * nb; i += blockDim.x) part[(size_t)blockIdx.x * 2 * nb + i] = sb[i];
 }
 
+// Column b of nblk partial rows of `pitch` doubles, summed by a warp in a fixed order
+// (on every lane).  One thread per bin took 45 us for 608 rows: a chain of loads.
+__device__ __forceinline__ double warp_column_sum(const double* col, int nblk, int pitch) {
+  double s = 0.0;
+  for (int i = threadIdx.x & 31; i < nblk; i += 32) s += col[(size_t)i * pitch];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
 __global__ void geo_final_kernel(const double* part, int nblk, int nb, double* geo) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // a warp per bin
   if (b >= nb) return;
-  double sn = 0.0, sc = 0.0;
-  for (int i = 0; i < nblk; ++i) {
-    sn += part[(size_t)i * 2 * nb + b];
-    sc += part[(size_t)i * 2 * nb + nb + b];
-  }
+  const double sn = warp_column_sum(part + b, nblk, 2 * nb), sc = warp_column_sum(part + nb + b, nblk, 2 * nb);
+  if (threadIdx.x & 31) return;
   geo[b] = sn;
   geo[nb + b] = sc;
 }
@@ -660,9 +838,12 @@ __global__ void geo_final_kernel(const double* part, int nblk, int nb, double* g
 // Shell sums of |F|^2 of a half spectrum with the cached bins: each kept mode
 // counts twice for 0 < kx < N/2 (its conjugate partner), runs of equal bins
 // along kx are summed before the atomic.  Partial rows of nb per block.
-__global__ void bin_power_half_kernel(const double2* H, const int* bin_of, int N, int nb, double* part) {
-  extern __shared__ double sb[];
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) sb[i] = 0.0;
+__global__ void bin_power_half_kernel(const double2* H, const int* bin_of, int N, int nb, int nc, double* part) {
+  extern __shared__ double sb_all[];
+  for (int i = threadIdx.x; i < nc * nb; i += blockDim.x) sb_all[i] = 0.0;
+  // nc copies of the bins, a warp adds to one of them: an FP64 addition to shared memory is
+  // repeated while others change the same word (256^3: 203 us with 32 warps to a copy, 116 us with 8)
+  double* const sb = sb_all + (threadIdx.x >> 5) % nc * nb;
   __syncthreads();
   constexpr int CH = 8;
   const int NH = N / 2 + 1, nchr = (NH + CH - 1) / CH;
@@ -674,33 +855,46 @@ __global__ void bin_power_half_kernel(const double2* H, const int* bin_of, int N
     const int y = (int)(row % N), z = (int)(row / N);
     const int ny = y <= N / 2 ? y : y - N, nz = z <= N / 2 ? z : z - N;
     const int c2 = ny * ny + nz * nz;
-    const int x1 = x0 + CH < NH ? x0 + CH : NH;
+    // runs of equal bins, two FP64 operations per mode; the columns between 0 and N/2
+    // stand for their partners too, the two edge columns are added once, apart
     int cur = -1;
     double rp = 0.0;
-    for (int kx = x0; kx < x1; ++kx) {
+    double2 v[CH];
+#pragma unroll
+    for (int i = 0; i < CH; ++i) v[i] = x0 + i < NH ? H[row * NH + x0 + i] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+      const int kx = x0 + i;
+      if (kx >= NH) break;
       const int b = bin_of[kx * kx + c2];
-      if (b < 0) continue;
+      if (kx == 0 || kx == N / 2) {
+        if (b >= 0) atomicAdd(&sb[b], fma(v[i].x, v[i].x, v[i].y * v[i].y));
+        continue;
+      }
       if (b != cur) {
-        if (cur >= 0) atomicAdd(&sb[cur], rp);
+        if (cur >= 0) atomicAdd(&sb[cur], 2.0 * rp);
         cur = b;
         rp = 0.0;
       }
-      const double2 v = H[row * NH + kx];
-      rp += ((kx == 0 || kx == N / 2) ? 1.0 : 2.0) * (v.x * v.x + v.y * v.y);
+      rp = fma(v[i].x, v[i].x, fma(v[i].y, v[i].y, rp));
     }
-    if (cur >= 0) atomicAdd(&sb[cur], rp);
+    if (cur >= 0) atomicAdd(&sb[cur], 2.0 * rp);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) part[(size_t)blockIdx.x * nb + i] = sb[i];
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    double t = 0.0;
+    for (int c = 0; c < nc; ++c) t += sb_all[c * nb + i];
+    part[(size_t)blockIdx.x * nb + i] = t;
+  }
 }
 
 // eq. discretePS per bin from the power rows and the cached geometry (as bin_final_kernel).
 __global__ void bin_final_geo_kernel(const double* part, int nblk, int nb, const double* geo, double kIR, double dx,
                                      int N, double* k, double* delta, double* mult) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // a warp per bin
   if (b >= nb) return;
-  double sp = 0.0;
-  for (int i = 0; i < nblk; ++i) sp += part[(size_t)i * nb + b];
+  const double sp = warp_column_sum(part + b, nblk, nb);
+  if (threadIdx.x & 31) return;
   const double sn = geo[b], sc = geo[nb + b];
   if (sc == 0.0) {
     k[b] = 0.0;
@@ -793,31 +987,58 @@ cudaError_t launch_ic_assemble(int fp32, void* phi, void* pi, const double2* F, 
   return cudaGetLastError();
 }
 
-// Lines per CTA: the largest divisor of N with batch * N <= 2048 (at most 72 KB
-// of shared memory per CTA).
-int fft_batch(int N) {
-  int b = 1;
-  for (int d = 1; d <= N && d * N <= 2048; ++d)
-    if (N % d == 0) b = d;
-  return b;
+// The plan of a transform along one axis of an array of x extent `pitch` (nu lines kept
+// along the fastest other index).
+FftPlan fft_plan(int N, int sign, const int4* tw, int pitch, int nu) {
+  FftPlan pl = {};
+  pl.N = N;
+  pl.sign = sign;
+  pl.batch = fft_batch_of(N);
+  pl.tw = tw;
+  pl.pitch = pitch;
+  pl.nu = nu;
+  pl.ng = (nu + pl.batch - 1) / pl.batch;
+  int Ns = 1;
+  for (int R : {4, 2, 3})
+    for (int m = N / Ns; m % R == 0; m /= R) {
+      FftStage& st = pl.st[pl.nrad++];
+      st.R = R;
+      st.Ns = Ns;
+      st.ts = N / (Ns * R);
+      st.NR = fast_div(N / R);
+      st.dNs = fast_div(Ns);
+      Ns *= R;
+    }
+  pl.dN = fast_div(N);
+  pl.dB = fast_div(pl.batch);
+  pl.dH = fast_div(N / 2 + 1);
+  pl.dg = fast_div(pl.ng);
+  return pl;
 }
 
-size_t fft_smem_bytes(int N) { return (2 * (size_t)fft_batch(N) * (N + 1) + N) * sizeof(double2); }
+size_t fft_smem_bytes(int N) {
+  const size_t B = (size_t)fft_batch_of(N);
+  return (2 * B * (N + 1) + N) * sizeof(CFix) + (B * (2 * sizeof(int) + sizeof(LineScale)) + 15) / 16 * 16;
+}
+// Threads per CTA: batch N <= 2048 elements, at most FFT_HELD a thread.
+int fft_threads(int N) { return std::max(64, (fft_batch_of(N) * N / FFT_HELD + 31) / 32 * 32); }
 
-cudaError_t launch_fft_twiddles(double2* tw, int N, cudaStream_t st) {
-  fft_twiddle_kernel<<<(N + 127) / 128, 128, 0, st>>>(tw, N);
+cudaError_t launch_fft_twiddles(int4* tw, int N, int sign, cudaStream_t st) {
+  fft_twiddle_kernel<<<(N + 127) / 128, 128, 0, st>>>(tw, N, sign);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fft_axis(double2* data, const FftPlan& pl, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute((const void*)fft_lines_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  void (*kern)(double2*, const FftPlan) = pl.N == 128   ? fft_lines_kernel<128>
+                                          : pl.N == 256 ? fft_lines_kernel<256>
+                                          : pl.N == 512 ? fft_lines_kernel<512>
+                                                        : fft_lines_kernel<0>;
+  cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)fft_smem_bytes(pl.N));
   if (e != cudaSuccess) return e;
-  const int work = pl.batch * pl.N / 4;
-  const int threads = work < 64 ? 64 : (work > 512 ? 512 : (work + 31) / 32 * 32);
-  const long long ng = pl.axis == 0 ? pl.N / pl.batch : (pl.nu + pl.batch - 1) / pl.batch;
-  const unsigned grid = (unsigned)(ng * pl.N);
-  fft_lines_kernel<<<grid, threads, fft_smem_bytes(pl.N), st>>>(data, pl);
+  const int threads = fft_threads(pl.N);
+  const unsigned grid = (unsigned)pl.ng * (unsigned)pl.N;
+  kern<<<grid, threads, fft_smem_bytes(pl.N), st>>>(data, pl);
   return cudaGetLastError();
 }
 
@@ -836,7 +1057,7 @@ cudaError_t launch_shell_geometry(int N, double dk, int nb, int nblk, int* bin_o
   geo_partial_kernel<<<nblk, 128, 2 * nb * sizeof(double), st>>>(bin_of, N, nb, part);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  geo_final_kernel<<<(nb + 127) / 128, 128, 0, st>>>(part, nblk, nb, geo);
+  geo_final_kernel<<<(nb + 3) / 4, 128, 0, st>>>(part, nblk, nb, geo);
   return cudaGetLastError();
 }
 
@@ -845,28 +1066,35 @@ cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftP
                                  const int* bin_of, const double* geo) {
   const int N = pl.N;
   cudaError_t e;
-  const void* kern = fp32 ? (const void*)rfft_rows_kernel<float> : (const void*)rfft_rows_kernel<double>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem_bytes(N));
+  auto rows = [&](auto kern, auto* src) -> cudaError_t {
+    const cudaError_t r = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)fft_smem_bytes(N));
+    if (r != cudaSuccess) return r;
+    kern<<<(unsigned)((long long)N * N / 2 / pl.batch), fft_threads(N), fft_smem_bytes(N), st>>>(src, H, pl);
+    return cudaGetLastError();
+  };
+  if (fp32) {
+    const float* src = (const float*)f;
+    e = N == 128   ? rows(rfft_rows_kernel<float, 128>, src)
+        : N == 256 ? rows(rfft_rows_kernel<float, 256>, src)
+        : N == 512 ? rows(rfft_rows_kernel<float, 512>, src)
+                   : rows(rfft_rows_kernel<float, 0>, src);
+  } else {
+    e = rows(rfft_rows_kernel<double, 0>, (const double*)f);
+  }
   if (e != cudaSuccess) return e;
-  const int work = pl.batch * N / 4;
-  const int threads = work < 64 ? 64 : (work > 512 ? 512 : (work + 31) / 32 * 32);
-  const unsigned grid = (unsigned)((long long)N * N / 2 / pl.batch);
-  if (fp32) rfft_rows_kernel<float><<<grid, threads, fft_smem_bytes(N), st>>>((const float*)f, H, pl);
-  else rfft_rows_kernel<double><<<grid, threads, fft_smem_bytes(N), st>>>((const double*)f, H, pl);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  FftPlan ph = pl;
-  ph.pitch = ph.nu = N / 2 + 1;
+  FftPlan ph = fft_plan(N, pl.sign, pl.tw, N / 2 + 1, N / 2 + 1);
   for (int axis = 1; axis < 3; ++axis) {
     ph.axis = axis;
     e = launch_fft_axis(H, ph, st);
     if (e != cudaSuccess) return e;
   }
   if (bin_of && geo) {  // the cached shell geometry: only the power is summed
-    bin_power_half_kernel<<<nblk, 256, nb * sizeof(double), st>>>(H, bin_of, N, nb, part);
+    const int nc = std::max(1, std::min(16, (int)(48 * 1024 / (nb * sizeof(double)))));
+    bin_power_half_kernel<<<nblk, 512, nc * nb * sizeof(double), st>>>(H, bin_of, N, nb, nc, part);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    bin_final_geo_kernel<<<(nb + 127) / 128, 128, 0, st>>>(part, nblk, nb, geo, kIR, dx, N, out, out + nb,
+    bin_final_geo_kernel<<<(nb + 3) / 4, 128, 0, st>>>(part, nblk, nb, geo, kIR, dx, N, out, out + nb,
                                                             out + 2 * nb);
     return cudaGetLastError();
   }
