@@ -24,7 +24,7 @@ namespace clg {
 template <typename T>
 __global__ void seed_chi_fraction_kernel(const LatConst* Lc, const LatScalars* Sc, int parity, T* lphi0,
                                          T* lpi0, T* lphi1, T* lpi1, double* part) {
-  __shared__ double red[256 / 32];
+  __shared__ double red[512 / 32];
   const LatConst& L = *Lc;
   const LatScalars& S = *Sc;
   const int N = L.N;
@@ -32,6 +32,8 @@ __global__ void seed_chi_fraction_kernel(const LatConst* Lc, const LatScalars* S
   const double rho = S.obs.rho, J = (S.obs.EK[1] + S.obs.EG[1]) / rho;
   const double a = S.a, a2 = a * a, a6 = a2 * a2 * a2;
   const double kK = 1.0 / (a6 * (double)V * rho), kG = -L.inv_dx2 / (a2 * (double)V), q = L.q;
+  // divisions once, not per site (about ten FP64 operations each)
+  const double iV = 1.0 / (double)V, irho = 1.0 / rho;
   const T* ph[2] = {reinterpret_cast<const T*>(L.buf[parity][0]), reinterpret_cast<const T*>(L.buf[parity][2])};
   const T* pm[2] = {reinterpret_cast<const T*>(L.buf[parity][1]), reinterpret_cast<const T*>(L.buf[parity][3])};
   T* lf[2] = {lphi0, lphi1};
@@ -53,7 +55,7 @@ __global__ void seed_chi_fraction_kernel(const LatConst* Lc, const LatScalars* S
       const double dEG = kG * lap;
       const double chi = g == 1 ? 1.0 : 0.0;
       lp[g][n] = (T)((chi - J) * (double)pm[g][n] * kK);
-      lf[g][n] = (T)((chi * dEG - J * (dEG + d[g] / (double)V)) / rho);
+      lf[g][n] = (T)((chi * dEG - J * (dEG + d[g] * iV)) * irho);
     }
     s += 0.5 * f0 * f0 * f1 * f1;
   }
@@ -126,10 +128,10 @@ cudaError_t launch_seed_chi_fraction(int fp32, const LatConst* L, LatScalars* S,
                                      void* const* lam, double* part, int nblk, double* out,
                                      cudaStream_t st) {
   if (fp32)
-    seed_chi_fraction_kernel<float><<<nblk, 256, 0, st>>>(L, S, parity, (float*)lam[0], (float*)lam[1],
+    seed_chi_fraction_kernel<float><<<nblk, 512, 0, st>>>(L, S, parity, (float*)lam[0], (float*)lam[1],
                                                           (float*)lam[2], (float*)lam[3], part);
   else
-    seed_chi_fraction_kernel<double><<<nblk, 256, 0, st>>>(L, S, parity, (double*)lam[0], (double*)lam[1],
+    seed_chi_fraction_kernel<double><<<nblk, 512, 0, st>>>(L, S, parity, (double*)lam[0], (double*)lam[1],
                                                            (double*)lam[2], (double*)lam[3], part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

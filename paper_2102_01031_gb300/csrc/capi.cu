@@ -1056,12 +1056,14 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
     double2* G = c->d_cplx + H.V;
     for (int f = 0; f < c->nf; ++f) {
       CU(cudaMemsetAsync(c->d_cplx, 0, 2 * (size_t)H.V * sizeof(double2), c->stream));
-      CU(launch_ic_modes(F, G, dL, dS, A, f, H.V, c->stream));
-      ++c->launches;
-      cl_status s = fft3d(c, H.N, F, +1);
-      if (s != CL_OK) return s;
-      s = fft3d(c, H.N, G, +1);
-      if (s != CL_OK) return s;
+      if (!(A.amp2 <= 0.0)) {  // without fluctuations every mode is zero, and so is its transform
+        CU(launch_ic_modes(F, G, dL, dS, A, f, H.V, c->stream));
+        ++c->launches;
+        cl_status s = fft3d(c, H.N, F, +1);
+        if (s != CL_OK) return s;
+        s = fft3d(c, H.N, G, +1);
+        if (s != CL_OK) return s;
+      }
       CU(launch_ic_assemble(c->fp32, arr_ptr(c, l, 0, 2 * f), arr_ptr(c, l, 0, 2 * f + 1), F, G, dL, dS,
                             c->p.phi0[f], c->p.dphi0[f], H.V, c->stream));
       ++c->launches;
@@ -1246,12 +1248,14 @@ static cl_status su2_init(cl_ctx* c, int N, double kIR, uint64_t seed) {
   // which start at zero homogeneous values
   for (int f = 0; f < (full ? 7 : 4); ++f) {
     CU(cudaMemsetAsync(c->d_cplx, 0, 2 * (size_t)H.V * sizeof(double2), c->stream));
-    CU(launch_ic_modes(F, G, c->d_lat, c->d_sc, A, f, H.V, c->stream));
-    ++c->launches;
-    cl_status s = fft3d(c, N, F, +1);
-    if (s != CL_OK) return s;
-    s = fft3d(c, N, G, +1);
-    if (s != CL_OK) return s;
+    if (!(A.amp2 <= 0.0)) {  // without fluctuations every mode is zero, and so is its transform
+      CU(launch_ic_modes(F, G, c->d_lat, c->d_sc, A, f, H.V, c->stream));
+      ++c->launches;
+      cl_status s = fft3d(c, N, F, +1);
+      if (s != CL_OK) return s;
+      s = fft3d(c, N, G, +1);
+      if (s != CL_OK) return s;
+    }
     const int af = f < 4 ? f : (f == 4 ? 35 : 37 + (f - 5));
     const int ap = f < 4 ? 4 + f : (f == 4 ? 36 : 39 + (f - 5));
     CU(launch_ic_assemble(c->fp32, arr_ptr(c, 0, 0, af), arr_ptr(c, 0, 0, ap), F, G, c->d_lat, c->d_sc,
