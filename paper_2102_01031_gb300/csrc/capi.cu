@@ -45,6 +45,7 @@ cudaError_t launch_su2_rho(int fp32, const LatConst* L, int parity, int g, doubl
 cudaError_t launch_su2_gauss_monitor(int fp32, const LatConst* L, int parity, double* part, int nblk,
                                      long long V, cudaStream_t st);
 constexpr int SU2_PARTIALS = 30;  // partial sums per CTA of the doublet-model pass
+constexpr int SU2_RED_ALPHA1 = 3; // its step passes at alpha = 1 (su2_common.cuh)
 
 cudaError_t launch_init_scalars(const LatConst*, LatScalars*, const ICArgs&, cudaStream_t);
 cudaError_t launch_ic_modes(double2*, double2*, const LatConst*, const LatScalars*, const ICArgs&,
@@ -306,7 +307,7 @@ PassKernel pick_kernel(const cl_ctx* c, int red) {
   if (is_doublet(c->model)) {
     const int full = c->model == CL_MODEL_LPHI4_SU2U1;
     if (su2_kd(c, red)) return su2_kd_pass_kernel(c->fp32, red, c->su2_tx, kd_ty(c, red), full, kd_n256(c, red));
-    return su2_pass_kernel(c->fp32, red, c->su2_tx, full);
+    return su2_pass_kernel(c->fp32, red == 1 && c->alpha == 1.0 ? SU2_RED_ALPHA1 : red, c->su2_tx, full);
   }
   // without self-consistent expansion the U(1) passes drift right after their
   // kick (the drift coefficient does not wait for the pass's sums)
@@ -1145,8 +1146,9 @@ static cl_status su2_init(cl_ctx* c, int N, double kIR, uint64_t seed) {
   int smax = 0;
   CU(cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->dev));
   for (int red = 0; red < 3; ++red) {
-    CU(cudaFuncSetAttribute((const void*)su2_pass_kernel(c->fp32, red, c->su2_tx, full),
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_bytes));
+    if (!su2_kd(c, red) && red != 0)
+      CU(cudaFuncSetAttribute((const void*)pick_kernel(c, red), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)c->smem_bytes));
     if (red != 1) {
       const int ty = kd_ty(c, red);
       const size_t sm = su2_kd_smem_bytes(c->su2_tx, ty, c->esz, full);

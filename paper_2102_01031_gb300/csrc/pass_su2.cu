@@ -38,7 +38,7 @@
 // into L1 while the next plane loads.  The two CTAs of an SM overlap one's
 // loads with the other's arithmetic.  The last CTA to finish sums the per-CTA
 // partial sums in a fixed order and advances the scale factor (tail.cuh).
-#include "su2_common.cuh"
+#include "su2_kick.cuh"
 
 namespace clg {
 
@@ -48,7 +48,8 @@ __host__ __device__ constexpr size_t su2_slot_bytes(int TX, int TY, int esz, boo
   return ((full ? 22 : 19) * (size_t)(TX + 2) * (TY + 2) * esz + 127) / 128 * 128;
 }
 
-// RED: 0 = no sums, 1 = sums for the Friedmann kicks, 2 = full measurement.
+// RED: 1 = sums for the Friedmann kicks, SU2_RED_ALPHA1 = the same at alpha = 1 (no gauge
+// energies), 2 = full measurement.
 // FULL: the lphi4SU2U1 model (Sec. 4.5): also a singlet phi_s and a U(1)-charged
 // scalar vphi (charge Qc in units of the doublet's, hopping with exp(-i Qc gQ dx A_i)),
 // coupled through V = lam (|Phi|^2 - v^2)^2 + qG |Phi|^2 phi_s^2 + 2 qH |Phi|^2 |vphi|^2:
@@ -58,7 +59,7 @@ __host__ __device__ constexpr size_t su2_slot_bytes(int TX, int TY, int esz, boo
 //   pi_A,i gains a^{1+alpha} (f_s/omega_s)^2 Qc (gQ/dx) (vphi_0 u_1 - vphi_1 u_0), u = its hop.
 template <typename T, int RED, int TX, bool FULL>
 __global__ void __launch_bounds__(256, (RED == 2 || sizeof(T) == 8) ? 1 : 2) dk_pass_su2(const PassArgs P) {
-  constexpr int NACC = RED == 0 ? 1 : (RED == 1 ? 6 : (FULL ? 29 : 23));
+  constexpr int NACC = RED == 1 ? 6 : (RED == SU2_RED_ALPHA1 ? 3 : (FULL ? 29 : 23));
   constexpr int NLD = FULL ? SNARR_FULL : SNARR;  // arrays loaded per halo site
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double red_s[SU2_NQ][9];
@@ -76,35 +77,18 @@ __global__ void __launch_bounds__(256, (RED == 2 || sizeof(T) == 8) ? 1 : 2) dk_
   T* const dst = reinterpret_cast<T*>(L.buf[parity ^ 1][0]);
   constexpr size_t slot_b = su2_slot_bytes(TX, TY, sizeof(T), FULL);
 
-  // coefficients: FP64 products by one lane, broadcast in the storage precision
-  T cf[17];
+  // the deferred drift and the kick's coefficients
+  T drift[3];
   if (lane == 0) {
-    const LatScalars* SC = P.sc;
-    const double ck = P.ck, ap1 = __ldcg(&SC->apow1), apm1 = __ldcg(&SC->apowm1);
-    const double cdA = __ldcg(&SC->cdA), dx = L.dx;
-    cf[0] = (T)__ldcg(&SC->cd);
-    cf[1] = (T)cdA;
-    cf[2] = (T)(0.5 * L.gQB * dx * cdA);                        // half the SU(2) drift angle per momentum
-    cf[3] = (T)(ck * ap1 * L.inv_dx2);                           // doublet Laplacian
-    cf[4] = (T)(ck * __ldcg(&SC->apow3));                        // potential force
-    cf[5] = (T)(ck * ap1 * L.fo2 * L.gQ / dx);                   // U(1) current
-    cf[6] = (T)(L.gQ != 0.0 ? -ck * apm1 / (L.gQ * dx * dx * dx) : 0.0);  // U(1) curl
-    cf[7] = (T)(ck * ap1 * L.fo2 * L.gQB / (2.0 * dx));          // SU(2) current
-    cf[8] = (T)(-2.0 * ck * apm1 / (L.gQB * dx * dx * dx));      // SU(2) plaquette force
-    cf[9] = (T)(L.gQ * dx);
-    cf[10] = (T)(L.v * L.v);
-    cf[11] = (T)L.lam;
-    cf[12] = (T)(2.0 * L.lam);
-    cf[13] = (T)L.qG;
-    cf[14] = (T)L.qH;
-    cf[15] = (T)(L.Qc * L.gQ * dx);                              // vphi's link phase per A_i
-    cf[16] = (T)(ck * ap1 * L.fo2 * L.Qc * L.gQ / dx);            // vphi's U(1) current
+    const double cdA64 = __ldcg(&P.sc->cdA);
+    drift[0] = (T)__ldcg(&P.sc->cd);
+    drift[1] = (T)cdA64;
+    drift[2] = (T)(0.5 * L.gQB * L.dx * cdA64);  // half the SU(2) drift angle per momentum
   }
 #pragma unroll
-  for (int k = 0; k < 17; ++k) cf[k] = __shfl_sync(0xffffffffu, cf[k], 0);
-  const T cd = cf[0], cdA = cf[1], hB = cf[2], A1 = cf[3], A3 = cf[4], AJA = cf[5], ACA = cf[6], AJB = cf[7],
-          AMB = cf[8], gd = cf[9], v2 = cf[10], lam = cf[11], lam2 = cf[12], qG = cf[13], qH = cf[14],
-          gdc = cf[15], AJC = cf[16];
+  for (int k = 0; k < 3; ++k) drift[k] = __shfl_sync(0xffffffffu, drift[k], 0);
+  const T cd = drift[0], cdA = drift[1], hB = drift[2];
+  const Su2Coef<T> cf = su2_coefficients<T>(L, P.sc, P.ck, lane);
   const bool drifting = cd != T(0) || cdA != T(0);
 
   Acc<T> acc[NACC];
@@ -223,11 +207,34 @@ __global__ void __launch_bounds__(256, (RED == 2 || sizeof(T) == 8) ? 1 : 2) dk_
     __syncthreads();  // the previous item's reads of the ring are done
     load_plane(0, x0, y0, (z0 - 1 + N) % N, false);
     load_plane(1, x0, y0, z0, true);
-    const int hx = tx + 1, hy = ty + 1, own = hy * HX + hx;
+    __syncthreads();
+    const int own = (ty + 1) * HX + tx + 1;
     const long long gown = (long long)(y0 + ty) * N + x0 + tx;
+    // the site's neighbourhood in slots s and s + 1 of the ring (su2_kick.cuh), its momenta
+    // from global memory (prefetched into L1)
+    struct Hood {
+      const unsigned char *c, *p;
+      const T* src;
+      long long g, V;
+      int own;
+      __device__ __forceinline__ const unsigned char* slot(int pl) const { return pl ? p : c; }
+      __device__ __forceinline__ Q4<T> u(int pl, int i, int dx, int dy) const {
+        return reinterpret_cast<const Q4<T>*>(slot(pl))[i * HS + own + dy * HX + dx];
+      }
+      __device__ __forceinline__ Q4<T> f(int pl, int dx, int dy) const { return u(pl, 3, dx, dy); }
+      __device__ __forceinline__ T a(int pl, int i, int dx, int dy) const {
+        return reinterpret_cast<const T*>(slot(pl))[(16 + i) * HS + own + dy * HX + dx];
+      }
+      __device__ __forceinline__ T x(int pl, int k, int dx, int dy) const { return a(pl, 3 + k, dx, dy); }
+      __device__ __forceinline__ T mom(int arr) const { return __ldg(src + arr * V + g); }
+    };
+    auto hood = [&](int s, long long g) {
+      return Hood{smem + s % 3 * slot_b, smem + (s + 1) % 3 * slot_b, src, g, V, own};
+    };
+    Su2Carry<T> carry = {};
+    su2_carry<T, FULL>(hood(0, 0), cf, carry);
     for (int j = 0; j < nz; ++j) {
       const int z = z0 + j;
-      const int sm = j % 3, sc = (j + 1) % 3, sp = (j + 2) % 3;
       const long long g = (long long)z * NN + gown;
       {  // the kick's own momenta move into L1 while the next plane loads
         const T* pp = src + g;
@@ -245,229 +252,29 @@ __global__ void __launch_bounds__(256, (RED == 2 || sizeof(T) == 8) ? 1 : 2) dk_
           prefetch_l1(pp + (SPC + 1) * V);
         }
       }
-      load_plane(sp, x0, y0, (z + 1) % N, j + 1 < nz);
+      // plane z + 1 into the slot that held z - 1: its values live on in the carries, and a
+      // warp that is still at the kick of z reads the other two slots, so that one barrier
+      // a plane is enough
+      load_plane((j + 2) % 3, x0, y0, (z + 1) % N, j + 1 < nz);
       __syncthreads();
-      // neighbours in the ring: (dx, dy) in the plane, slot for dz
-      auto at = [&](int ddx, int ddy) { return own + ddy * HX + ddx; };
-      const Q4<T> psi = sF(sc)[own];
-      Q4<T> D;
-      D.w = T(-6) * psi.w;
-      D.x = T(-6) * psi.x;
-      D.y = T(-6) * psi.y;
-      D.z = T(-6) * psi.z;
-      T s_g = T(0), s_pA = T(0), s_pB = T(0), s_mA = T(0), s_mB = T(0);
-      T pnA[3], pnB[3][3];
-      // FULL: the singlet's Laplacian and gradient sum, vphi's covariant Laplacian and gradient sum
-      T xs0 = T(0), xc0 = T(0), xc1 = T(0), Ls = T(0), Dv0 = T(0), Dv1 = T(0), s_gs = T(0), s_gc = T(0);
-      if constexpr (FULL) {
-        xs0 = sX(sc, 0)[own];
-        xc0 = sX(sc, 1)[own];
-        xc1 = sX(sc, 2)[own];
-        Ls = T(-6) * xs0;
-        Dv0 = T(-6) * xc0;
-        Dv1 = T(-6) * xc1;
-      }
-      // U(1) plaquette sines: xy, xz, yz at n, then the lower ones
-      const T ax = sA(sc, 0)[own], ay = sA(sc, 1)[own], az = sA(sc, 2)[own];
-      T sxy = T(0), sxz = T(0), syz = T(0), Cx = T(0), Cy = T(0), Cz = T(0);
-      if (ACA != T(0) || RED > 0) {
-        const T txy = gd * ((ax + sA(sc, 1)[at(1, 0)]) - (sA(sc, 0)[at(0, 1)] + ay));
-        const T txz = gd * ((ax + sA(sc, 2)[at(1, 0)]) - (sA(sp, 0)[own] + az));
-        const T tyz = gd * ((ay + sA(sc, 2)[at(0, 1)]) - (sA(sp, 1)[own] + az));
-        sxy = sin_t(txy);
-        sxz = sin_t(txz);
-        syz = sin_t(tyz);
-        const T sxy_ym = sin_t(gd * ((sA(sc, 0)[at(0, -1)] + sA(sc, 1)[at(1, -1)]) - (ax + sA(sc, 1)[at(0, -1)])));
-        const T sxy_xm = sin_t(gd * ((sA(sc, 0)[at(-1, 0)] + ay) - (sA(sc, 0)[at(-1, 1)] + sA(sc, 1)[at(-1, 0)])));
-        const T sxz_zm = sin_t(gd * ((sA(sm, 0)[own] + sA(sm, 2)[at(1, 0)]) - (ax + sA(sm, 2)[own])));
-        const T sxz_xm = sin_t(gd * ((sA(sc, 0)[at(-1, 0)] + az) - (sA(sp, 0)[at(-1, 0)] + sA(sc, 2)[at(-1, 0)])));
-        const T syz_zm = sin_t(gd * ((sA(sm, 1)[own] + sA(sm, 2)[at(0, 1)]) - (ay + sA(sm, 2)[own])));
-        const T syz_ym = sin_t(gd * ((sA(sc, 1)[at(0, -1)] + az) - (sA(sp, 1)[at(0, -1)] + sA(sc, 2)[at(0, -1)])));
-        Cx = (sxy - sxy_ym) + (sxz - sxz_zm);
-        Cy = (sxy_xm - sxy) + (syz - syz_zm);
-        Cz = (sxz_xm - sxz) + (syz_ym - syz);
-        if constexpr (RED > 0) {
-          const T hx2 = sin_t(T(0.5) * txy), hy2 = sin_t(T(0.5) * txz), hz2 = sin_t(T(0.5) * tyz);
-          s_mA = T(2) * (hx2 * hx2 + hy2 * hy2 + hz2 * hz2);
-        }
-      }
-      const T Cc[3] = {Cx, Cy, Cz};
+      auto link = [&](int i, const Q4<T>&, T, T pnA, const T (&pnB)[3]) {
+        if (!P.write) return;
+        dst[(SPA + i) * V + g] = pnA;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        // ---- doublet hops along i, currents ----
-        const Q4<T> Ui = sU(sc, i)[own];
-        const int fx = i == 0 ? 1 : 0, fy = i == 1 ? 1 : 0;
-        const Q4<T> fn = i == 2 ? sF(sp)[own] : sF(sc)[at(fx, fy)];
-        Q4<T> chi = umul(Ui, fn);
-        T c, s;
-        sincos_t(gd * sA(sc, i)[own], s, c);
-        phase(chi, c, s);
-        const int bs = i == 2 ? sm : sc;
-        const int bk = i == 2 ? own : at(-fx, -fy);
-        Q4<T> back = udmul(sU(bs, i)[bk], sF(bs)[bk]);
-        sincos_t(gd * sA(bs, i)[bk], s, c);
-        phase(back, c, -s);
-        D.w += chi.w + back.w;
-        D.x += chi.x + back.x;
-        D.y += chi.y + back.y;
-        D.z += chi.z + back.z;
-        // psi = (p, q) = (w + i x, y + i z), chi = (c1, c2)
-        const T ImA = (psi.w * chi.x - psi.x * chi.w) + (psi.y * chi.z - psi.z * chi.y);     // Im psi^dag chi
-        const T Im1 = (psi.w * chi.z - psi.x * chi.y) + (psi.y * chi.x - psi.z * chi.w);     // Im psi^dag s1 chi
-        const T Im2 = (psi.y * chi.w + psi.z * chi.x) - (psi.w * chi.y + psi.x * chi.z);     // Im psi^dag s2 chi
-        const T Im3 = (psi.w * chi.x - psi.x * chi.w) - (psi.y * chi.z - psi.z * chi.y);     // Im psi^dag s3 chi
-        if constexpr (RED > 0) {
-          const T e0 = chi.w - psi.w, e1 = chi.x - psi.x, e2 = chi.y - psi.y, e3 = chi.z - psi.z;
-          s_g += (e0 * e0 + e1 * e1) + (e2 * e2 + e3 * e3);
-        }
-        // ---- SU(2) staples of U_i(n) ----
-        Q4<T> S;
-        S.w = S.x = S.y = S.z = T(0);
-#pragma unroll
-        for (int jj = 1; jj <= 2; ++jj) {
-          const int j = (i + jj) % 3;
-          const int gx = j == 0 ? 1 : 0, gy = j == 1 ? 1 : 0;
-          // U_j(n+i), U_i(n+j), U_j(n)
-          const Q4<T> ujni = i == 2 ? sU(sp, j)[own] : sU(sc, j)[at(fx, fy)];
-          const Q4<T> uinj = j == 2 ? sU(sp, i)[own] : sU(sc, i)[at(gx, gy)];
-          const Q4<T> ujn = sU(sc, j)[own];
-          const Q4<T> up = qmul(qmul(ujni, qconj(uinj)), qconj(ujn));
-          // U_j(n+i-j), U_i(n-j), U_j(n-j)
-          Q4<T> ujnimj, uinmj, ujnmj;
-          if (j == 2) {
-            ujnimj = i == 2 ? sU(sc, j)[own] : sU(sm, j)[at(fx, fy)];
-            uinmj = sU(sm, i)[own];
-            ujnmj = sU(sm, j)[own];
-          } else if (i == 2) {
-            ujnimj = sU(sp, j)[at(-gx, -gy)];
-            uinmj = sU(sc, i)[at(-gx, -gy)];
-            ujnmj = sU(sc, j)[at(-gx, -gy)];
-          } else {
-            ujnimj = sU(sc, j)[at(fx - gx, fy - gy)];
-            uinmj = sU(sc, i)[at(-gx, -gy)];
-            ujnmj = sU(sc, j)[at(-gx, -gy)];
-          }
-          const Q4<T> lo = qmul(qmul(qconj(ujnimj), qconj(uinmj)), ujnmj);
-          qadd(S, up);
-          qadd(S, lo);
-          if constexpr (RED > 0) {
-            if (j > i) s_mB += one_minus_w(qmul(Ui, up));
-          }
-        }
-        const Q4<T> M = qmul(Ui, S);
-        // ---- link kicks ----
-        const T pA = __ldg(src + (SPA + i) * V + g);
-        pnA[i] = pA + (AJA * ImA + ACA * Cc[i]);
-        if constexpr (FULL) {
-          // singlet neighbours along i
-          const T sfw = i == 2 ? sX(sp, 0)[own] : sX(sc, 0)[at(fx, fy)];
-          const T sbw = sX(bs, 0)[bk];
-          Ls += sfw + sbw;
-          // vphi: forward hop Vc_i(n) vphi(n+i), backward hop Vc_i^*(n-i) vphi(n-i), Vc = exp(-i Qc gQ dx A)
-          const T y0 = i == 2 ? sX(sp, 1)[own] : sX(sc, 1)[at(fx, fy)];
-          const T y1 = i == 2 ? sX(sp, 2)[own] : sX(sc, 2)[at(fx, fy)];
-          T cc, sc2;
-          sincos_t(gdc * sA(sc, i)[own], sc2, cc);
-          const T u0 = cc * y0 + sc2 * y1, u1 = cc * y1 - sc2 * y0;
-          const T b0 = sX(bs, 1)[bk], b1 = sX(bs, 2)[bk];
-          sincos_t(gdc * sA(bs, i)[bk], sc2, cc);
-          const T w0 = cc * b0 - sc2 * b1, w1 = cc * b1 + sc2 * b0;
-          Dv0 += u0 + w0;
-          Dv1 += u1 + w1;
-          pnA[i] += AJC * (xc0 * u1 - xc1 * u0);
-          if constexpr (RED > 0) {
-            const T gs = sfw - xs0, g0 = u0 - xc0, g1 = u1 - xc1;
-            s_gs += gs * gs;
-            s_gc += g0 * g0 + g1 * g1;
-          }
-        }
-        const T Ims[3] = {Im1, Im2, Im3};
-        const T Ms[3] = {M.x, M.y, M.z};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          const T pB = __ldg(src + (SPB + 3 * i + a) * V + g);
-          pnB[i][a] = pB + (AJB * Ims[a] + AMB * Ms[a]);
-        }
-        if constexpr (RED > 0) {
-          s_pA += pnA[i] * pnA[i];
-          s_pB += pnB[i][0] * pnB[i][0] + pnB[i][1] * pnB[i][1] + pnB[i][2] * pnB[i][2];
-        }
-      }
-      // ---- doublet kick ----
-      const T r2 = T(0.5) * ((psi.w * psi.w + psi.x * psi.x) + (psi.y * psi.y + psi.z * psi.z));
-      const T dd = r2 - v2;
-      T gp = lam2 * dd;
-      T c2v = T(0);  // FULL: |vphi|^2
-      if constexpr (FULL) {
-        c2v = T(0.5) * (xc0 * xc0 + xc1 * xc1);
-        gp += qG * xs0 * xs0 + T(2) * qH * c2v;
-      }
-      T pn[4];
-      const T Dc[4] = {D.w, D.x, D.y, D.z};
-      const T fc[4] = {psi.w, psi.x, psi.y, psi.z};
-#pragma unroll
-      for (int c2 = 0; c2 < 4; ++c2) pn[c2] = __ldg(src + (SP + c2) * V + g) + (A1 * Dc[c2] - A3 * gp * fc[c2]);
-      // FULL: kicks of the singlet and of vphi
-      T pns = T(0), pnc0 = T(0), pnc1 = T(0);
-      if constexpr (FULL) {
-        pns = __ldg(src + SPS * V + g) + (A1 * Ls - A3 * (T(2) * qG * r2) * xs0);
-        pnc0 = __ldg(src + SPC * V + g) + (A1 * Dv0 - A3 * (T(2) * qH * r2) * xc0);
-        pnc1 = __ldg(src + (SPC + 1) * V + g) + (A1 * Dv1 - A3 * (T(2) * qH * r2) * xc1);
-        if (P.write) {
-          dst[SPS * V + g] = pns;
-          dst[SPC * V + g] = pnc0;
-          dst[(SPC + 1) * V + g] = pnc1;
-        }
-      }
+        for (int a = 0; a < 3; ++a) dst[(SPB + 3 * i + a) * V + g] = pnB[a];
+      };
+      Su2Site<T> site;
+      su2_kick<T, RED, FULL>(hood(j + 1, g), cf, carry, site, [] {}, link);
       if (P.write) {
 #pragma unroll
-        for (int c2 = 0; c2 < 4; ++c2) dst[(SP + c2) * V + g] = pn[c2];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          dst[(SPA + i) * V + g] = pnA[i];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) dst[(SPB + 3 * i + a) * V + g] = pnB[i][a];
+        for (int c2 = 0; c2 < 4; ++c2) dst[(SP + c2) * V + g] = site.pn[c2];
+        if constexpr (FULL) {
+          dst[SPS * V + g] = site.pns;
+          dst[SPC * V + g] = site.pnc0;
+          dst[(SPC + 1) * V + g] = site.pnc1;
         }
       }
-      if constexpr (RED == 1) {
-        acc[0].add((pn[0] * pn[0] + pn[1] * pn[1]) + (pn[2] * pn[2] + pn[3] * pn[3]));
-        acc[1].add(s_pA + s_pB);
-        acc[2].add(s_g);
-        acc[3].add(s_mA);
-        acc[4].add(s_mB);
-        acc[5].add(lam * dd * dd);
-        if constexpr (FULL) {  // the Friedmann kick takes the totals
-          acc[0].add(pns * pns + (pnc0 * pnc0 + pnc1 * pnc1));
-          acc[2].add(s_gs + s_gc);
-          acc[5].add(qG * r2 * xs0 * xs0 + T(2) * qH * r2 * c2v);
-        }
-      } else if constexpr (RED == 2) {
-#pragma unroll
-        for (int c2 = 0; c2 < 4; ++c2) {
-          acc[c2].add(pn[c2] * pn[c2]);
-          acc[10 + c2].add(fc[c2]);
-          acc[14 + c2].add(fc[c2] * fc[c2]);
-          acc[18 + c2].add(pn[c2]);
-          if (!isfinite(pn[c2])) nonfinite += 1.f;
-        }
-        acc[4].add(s_pA);
-        acc[5].add(s_pB);
-        acc[6].add(s_g);
-        acc[7].add(s_mA);
-        acc[8].add(s_mB);
-        acc[9].add(lam * dd * dd);
-        if (!isfinite(s_pA) || !isfinite(s_pB)) nonfinite += 1.f;
-        if constexpr (FULL) {  // per species: singlet, vphi
-          acc[23].add(pns * pns);
-          acc[24].add(pnc0 * pnc0 + pnc1 * pnc1);
-          acc[25].add(s_gs);
-          acc[26].add(s_gc);
-          acc[27].add(qG * r2 * xs0 * xs0);
-          acc[28].add(T(2) * qH * r2 * c2v);
-          if (!isfinite(pns) || !isfinite(pnc0) || !isfinite(pnc1)) nonfinite += 1.f;
-        }
-      }
-      __syncthreads();  // slot sm is overwritten by the next load
+      su2_sums<T, RED, FULL>(cf, site, acc, nonfinite);
     }
   }
 
@@ -476,19 +283,21 @@ __global__ void __launch_bounds__(256, (RED == 2 || sizeof(T) == 8) ? 1 : 2) dk_
 
 typedef void (*PassKernel)(const PassArgs);
 
+// red: 1, 2 or SU2_RED_ALPHA1 (without self-consistent expansion the passes of pass_su2_kd.cu run).
 PassKernel su2_pass_kernel(int fp32, int red, int TX, int full) {
-  static const PassKernel tab[2][2][3] = {
-      {{dk_pass_su2<double, 0, 16, false>, dk_pass_su2<double, 1, 16, false>, dk_pass_su2<double, 2, 16, false>},
-       {dk_pass_su2<float, 0, 16, false>, dk_pass_su2<float, 1, 16, false>, dk_pass_su2<float, 2, 16, false>}},
-      {{dk_pass_su2<double, 0, 32, false>, dk_pass_su2<double, 1, 32, false>, dk_pass_su2<double, 2, 32, false>},
-       {dk_pass_su2<float, 0, 32, false>, dk_pass_su2<float, 1, 32, false>, dk_pass_su2<float, 2, 32, false>}}};
-  static const PassKernel tab_full[2][2][3] = {
-      {{dk_pass_su2<double, 0, 16, true>, dk_pass_su2<double, 1, 16, true>, dk_pass_su2<double, 2, 16, true>},
-       {dk_pass_su2<float, 0, 16, true>, dk_pass_su2<float, 1, 16, true>, dk_pass_su2<float, 2, 16, true>}},
-      {{dk_pass_su2<double, 0, 32, true>, dk_pass_su2<double, 1, 32, true>, dk_pass_su2<double, 2, 32, true>},
-       {dk_pass_su2<float, 0, 32, true>, dk_pass_su2<float, 1, 32, true>, dk_pass_su2<float, 2, 32, true>}}};
-  if (red < 0 || red > 2 || (TX != 16 && TX != 32)) return nullptr;
-  return (full ? tab_full : tab)[TX == 32 ? 1 : 0][fp32 ? 1 : 0][red];
+  constexpr int A1 = SU2_RED_ALPHA1;
+  static const PassKernel tab[2][2][2][3] = {  // [full][TX == 32][fp32][red - 1]
+      {{{dk_pass_su2<double, 1, 16, false>, dk_pass_su2<double, 2, 16, false>, dk_pass_su2<double, A1, 16, false>},
+        {dk_pass_su2<float, 1, 16, false>, dk_pass_su2<float, 2, 16, false>, dk_pass_su2<float, A1, 16, false>}},
+       {{dk_pass_su2<double, 1, 32, false>, dk_pass_su2<double, 2, 32, false>, dk_pass_su2<double, A1, 32, false>},
+        {dk_pass_su2<float, 1, 32, false>, dk_pass_su2<float, 2, 32, false>, dk_pass_su2<float, A1, 32, false>}}},
+      {{{dk_pass_su2<double, 1, 16, true>, dk_pass_su2<double, 2, 16, true>, dk_pass_su2<double, A1, 16, true>},
+        {dk_pass_su2<float, 1, 16, true>, dk_pass_su2<float, 2, 16, true>, dk_pass_su2<float, A1, 16, true>}},
+       {{dk_pass_su2<double, 1, 32, true>, dk_pass_su2<double, 2, 32, true>, dk_pass_su2<double, A1, 32, true>},
+        {dk_pass_su2<float, 1, 32, true>, dk_pass_su2<float, 2, 32, true>, dk_pass_su2<float, A1, 32, true>}}}};
+  static_assert(A1 == 3, "the table's order");
+  if (red < 1 || red > 3 || (TX != 16 && TX != 32)) return nullptr;
+  return tab[full ? 1 : 0][TX == 32 ? 1 : 0][fp32 ? 1 : 0][red - 1];
 }
 
 size_t su2_smem_bytes(int TX, int TY, int esz, int full) { return 3 * su2_slot_bytes(TX, TY, esz, full != 0); }

@@ -121,6 +121,8 @@ __device__ __forceinline__ T one_minus_w(const Q4<T>& p) {
   return (p.x * p.x + p.y * p.y + p.z * p.z) / (T(1) + p.w);
 }
 
+constexpr int SU2_RED_ALPHA1 = 3;  // a pass's sums at alpha = 1: the Friedmann kicks' without the gauge fields'
+
 constexpr int SU2_NQ = 30;  // partial sums per CTA (the measurement pass uses 23, 29 for lphi4SU2U1)
 
 constexpr int SU2_TY = 8;  // tile height of the passes; the width TX (32 or 16) is a template parameter
@@ -129,7 +131,7 @@ constexpr int SU2_TY = 8;  // tile height of the passes; the width TX (32 or 16)
 // into red_s, the CTA's slot of P.partials, and in the last CTA to arrive the
 // fixed-order lattice sums, the energies (RED 2), the scale-factor update and
 // the drift coefficients of the next pass.  RED: 0 no sums, 1 the Friedmann
-// kicks' sums, 2 a full measurement.
+// kicks' sums, 2 a full measurement, SU2_RED_ALPHA1 as 1 without the gauge fields'.
 template <typename T, int RED, bool FULL, int NACC>
 __device__ void su2_pass_end(const PassArgs& P, const LatConst& L, Acc<T> (&acc)[NACC], float nonfinite,
                              double (*red_s)[9], unsigned& last_s, int tid, int lane, int warp, int nth) {
@@ -189,6 +191,11 @@ __device__ void su2_pass_end(const PassArgs& P, const LatConst& L, Acc<T> (&acc)
       EGA = red_s[3][0] * mA;
       EGB = red_s[4][0] * mB;
       E.EV = red_s[5][0] * L.inv_V;
+    } else if (RED == SU2_RED_ALPHA1) {  // the gauge energies' factor alpha - 1 is zero
+      spost = red_s[0][0];
+      slinks = 0.0;
+      E.EG = red_s[1][0] * gphi;
+      E.EV = red_s[2][0] * L.inv_V;
     } else {
       spost = red_s[0][0] + red_s[1][0] + red_s[2][0] + red_s[3][0];
       slinks = red_s[4][0] + red_s[5][0];
