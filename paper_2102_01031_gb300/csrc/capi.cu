@@ -34,7 +34,7 @@ typedef void (*PassKernel)(const PassArgs);
 // the singlet and the U(1)-charged scalar of the lphi4SU2U1 example.
 inline bool is_doublet(int model) { return model == CL_MODEL_SU2U1_HIGGS || model == CL_MODEL_LPHI4_SU2U1; }
 PassKernel scalar_pass_kernel(int fp32, int nf, int red);
-PassKernel u1_pass_kernel(int fp32, int red, int kd, int n256);
+PassKernel u1_pass_kernel(int fp32, int red, int kd, int n256, int alpha1);
 PassKernel su2_pass_kernel(int fp32, int red, int TX, int full);
 size_t su2_smem_bytes(int TX, int TY, int esz, int full);
 PassKernel su2_kd_pass_kernel(int fp32, int red, int TX, int TY, int full, int n256);
@@ -313,7 +313,7 @@ PassKernel pick_kernel(const cl_ctx* c, int red) {
   // kick (the drift coefficient does not wait for the pass's sums)
   if (c->model == CL_MODEL_U1_HIGGS) {
     const bool n256 = c->nlat == 1 && c->lats[0].N == 256 && c->lats[0].BY == THREADS / (256 / u1_vx(c->esz));
-    return u1_pass_kernel(c->fp32, red, c->p.expansion != CL_EXP_SELF, n256);
+    return u1_pass_kernel(c->fp32, red, c->p.expansion != CL_EXP_SELF, n256, c->alpha == 1.0);
   }
   return scalar_pass_kernel(c->fp32, c->nf, red);
 }

@@ -36,6 +36,12 @@ namespace clg {
 
 namespace {
 
+// A step pass with self-consistent expansion at alpha = 1 forms no energies of the links: its
+// issue slots bound it (three of a site's sines and two of five FP64 sums go; 144^3 FP32,
+// 20 VV2 steps and energies 1821 -> 1599 us).  alpha is a context's constant, so the host
+// picks the kernel.
+constexpr int U1_RED_ALPHA1 = 3;
+
 enum : int { F0 = 0, P0 = 1, F1 = 2, P1 = 3, AX = 4, PAX = 5, AY = 6, PAY = 7, AZ = 8, PAZ = 9 };
 
 template <typename T> struct U1Vec;
@@ -146,8 +152,8 @@ struct U1Update {
     q->fast = 0;
     if (RED == 0) return;
     const LatPar& L = r->L;
-    if (RED == 1 && L.expansion == CL_EXP_SELF && L.int_alpha && L.alpha_i == 1) {
-      alpha1_ready(L, r->W, q);  // the links' energies enter with alpha - 1 = 0
+    if (RED == U1_RED_ALPHA1) {
+      alpha1_ready(L, r->W, q);
       return;
     }
     const double a = r->W.a, a2 = a * a, a4 = a2 * a2, a6 = a4 * a2;
@@ -159,14 +165,13 @@ struct U1Update {
     if (L.expansion == CL_EXP_SELF) q->pref = kernel_a_pref(L, a);
   }
   __device__ __noinline__ static void fast_drift(Rec* r, const TailPrep* q, const double* sum) {
-    alpha1_drift(r->W, q, alpha1_b(q, sum[0], sum[2], sum[4]));
+    alpha1_drift(r->W, q, alpha1_b(q, sum[0], sum[1], sum[2]));
     r->cf[0] = (T)r->W.cd;
     r->cf[1] = (T)r->W.cdA;
-    r->W.pi2 = sum[0];
-    r->W.pi2A = sum[1];
+    r->W.pi2 = sum[0];  // pi2A, which enters with alpha - 1 = 0, stays
   }
   __device__ __noinline__ static void fast_powers(Rec* r, const TailPrep* q, const double* sum, double*, double*) {
-    alpha1_powers(r->W, q, alpha1_b(q, sum[0], sum[2], sum[4]));
+    alpha1_powers(r->W, q, alpha1_b(q, sum[0], sum[1], sum[2]));
     const double k1 = q->ckn * r->W.apow1;
     r->cf[2] = (T)(k1 * r->L.inv_dx2);
     r->cf[3] = (T)(q->ckn * r->W.apow3);
@@ -179,7 +184,7 @@ struct U1Update {
     const PassStep st = {0.0, q->wout, q->win, q->dnext};
     ScalarState W = r->W;
     PassSums E = {0, 0, 0, 0, 0, 0, 0};
-    if (RED > 0) {
+    if (RED == 1 || RED == 2) {
       constexpr int o = RED == 1 ? 0 : 1;
       const double spost = RED == 1 ? sum[0] : sum[0] + sum[1];
       const double spA = sum[1 + o], gg = sum[2 + o], mag = sum[3 + o], vs = sum[4 + o];
@@ -235,7 +240,9 @@ struct U1Update {
 
 }  // namespace
 
-// RED: 0 = no sums, 1 = sums for the Friedmann kick, 2 = full measurement.
+// RED: 0 = no sums, 1 = sums for the Friedmann kick, 2 = full measurement, U1_RED_ALPHA1 =
+// the Friedmann kick's sums at alpha = 1, where the links' energies enter with alpha - 1 = 0
+// and are not formed (three half-angle sines a site and the momenta's squares).
 // KD: the pass's own drift follows its kick at each site (kick, then drift by
 // the pass's dnext), instead of being deferred to the next pass's reads.  The
 // order of operations on every value is the same; it needs the drift
@@ -253,9 +260,11 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
   typedef typename U1Vec<T>::type V;
   constexpr int NAR = 10;  // arrays in a ring stage
   // RED 1: pi_phi^2, pi_A^2, |D+ phi|^2, magnetic, V.
+  // U1_RED_ALPHA1: pi_phi^2, |D+ phi|^2, V.
   // RED 2: pi_0^2, pi_1^2, pi_A^2, |D+ phi|^2, magnetic, V, <phi_c>, <phi_c^2>, <pi_c>.
-  constexpr int NACC = RED == 0 ? 1 : (RED == 1 ? 5 : 12);
-  constexpr int NUSED = RED == 0 ? 0 : (RED == 1 ? 5 : NQ);
+  constexpr int NACC = RED == 0 ? 1 : (RED == 1 ? 5 : (RED == U1_RED_ALPHA1 ? 3 : 12));
+  constexpr int NUSED = RED == 0 ? 0 : (RED == 2 ? NQ : NACC);
+  constexpr bool GS = RED == 1 || RED == 2;  // the links' sums
 
   extern __shared__ __align__(128) unsigned char smem[];
   const Ring R = ring_view(smem, P);
@@ -449,7 +458,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
                 const T q0 = vget(pn0, v), q1 = vget(pn1, v), h0 = vget(f0, v), h1 = vget(f1, v), d = vget(dd, v);
                 s_g += e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3 + e4 * e4 + e5 * e5;
                 s_v += lam * d * d;
-                if constexpr (RED == 1) {
+                if constexpr (RED != 2) {
                   s_pi += q0 * q0 + q1 * q1;
                 } else {
                   acc[0].add(q0 * q0);
@@ -489,7 +498,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
             const V pnx = vadd(pax, vfma(AJv, Jx, vmul(ACv, Cx)));
             const V pny = vadd(pay, vfma(AJv, Jy, vmul(ACv, Cy)));
             const V pnz = vadd(paz, vfma(AJv, Jz, vmul(ACv, Cz)));
-            if constexpr (RED > 0) {
+            if constexpr (GS) {
               const V hxy = vsin(vmul(vset(T(0.5)), txy)), hxz = vsin(vmul(vset(T(0.5)), txz));
               const V hyz = vsin(vmul(vset(T(0.5)), tyz));
 #pragma unroll
@@ -517,7 +526,11 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
               stv(out + PAZ * Vs, pnz);
             }
           }
-          if constexpr (RED == 1) {
+          if constexpr (RED == U1_RED_ALPHA1) {
+            acc[0].add(s_pi);
+            acc[1].add(s_g);
+            acc[2].add(s_v);
+          } else if constexpr (RED == 1) {
             acc[0].add(s_pi);
             acc[1].add(s_piA);
             acc[2].add(s_g);
@@ -565,6 +578,8 @@ timeout:
 
 template __global__ void dk_pass_u1<float, 0, false, 0>(const __grid_constant__ PassArgs);
 template __global__ void dk_pass_u1<float, 1, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<float, U1_RED_ALPHA1, false, 0>(const __grid_constant__ PassArgs);
+template __global__ void dk_pass_u1<double, U1_RED_ALPHA1, false, 0>(const __grid_constant__ PassArgs);
 template __global__ void dk_pass_u1<float, 2, false, 0>(const __grid_constant__ PassArgs);
 template __global__ void dk_pass_u1<double, 0, false, 0>(const __grid_constant__ PassArgs);
 template __global__ void dk_pass_u1<double, 1, false, 0>(const __grid_constant__ PassArgs);
@@ -581,7 +596,8 @@ typedef void (*PassKernel)(const PassArgs);
 // kd: kick-then-drift passes (only without self-consistent expansion, where the
 // Friedmann sums of RED 1 are not needed).  n256: one FP32 lattice of N = 256 with full
 // tiles (the tile height THREADS / (N / 2)), built with its sizes as constants.
-PassKernel u1_pass_kernel(int fp32, int red, int kd, int n256) {
+// alpha1: self-consistent expansion with alpha = 1.
+PassKernel u1_pass_kernel(int fp32, int red, int kd, int n256, int alpha1) {
   static const PassKernel tab[2][3] = {
       {dk_pass_u1<double, 0, false, 0>, dk_pass_u1<double, 1, false, 0>, dk_pass_u1<double, 2, false, 0>},
       {dk_pass_u1<float, 0, false, 0>, dk_pass_u1<float, 1, false, 0>, dk_pass_u1<float, 2, false, 0>}};
@@ -591,6 +607,8 @@ PassKernel u1_pass_kernel(int fp32, int red, int kd, int n256) {
   static const PassKernel tab_kd256[3] = {dk_pass_u1<float, 0, true, 256>, nullptr,
                                           dk_pass_u1<float, 2, true, 256>};
   if (red < 0 || red > 2) return nullptr;
+  if (!kd && red == 1 && alpha1)
+    return fp32 ? dk_pass_u1<float, U1_RED_ALPHA1, false, 0> : dk_pass_u1<double, U1_RED_ALPHA1, false, 0>;
   if (kd && n256 && fp32) return tab_kd256[red];
   return kd ? tab_kd[fp32 ? 1 : 0][red] : tab[fp32 ? 1 : 0][red];
 }
