@@ -116,6 +116,7 @@ struct alignas(16) SegInfo {
 // Shared-memory layout behind the stage ring of a DK pass (byte offsets).
 constexpr size_t SM_FULL = 0;                                   // 8 mbarriers
 constexpr size_t SM_RELEASED = 64;                              // 8 release counts
+constexpr size_t SM_DRIFTED = 96;                               // mbarrier: a plane's values written back drifted (FP64 scalar pass)
 constexpr size_t SM_OFF = 128;                                  // MAX_SEG_PER_CTA + 1 plane offsets
 constexpr size_t SM_RED = (SM_OFF + 4 * (MAX_SEG_PER_CTA + 1) + 127) / 128 * 128;  // 33 x NQ doubles
 constexpr size_t SM_FLAG = SM_RED + 33 * NQ * 8;                // 4 ints + pending tails

@@ -24,9 +24,20 @@
 // (FP32) or plain (FP64) accumulators and flushed once per run into the run's
 // slot; between two passes every CTA sums its lattices' slots in a fixed order
 // and runs their Friedmann update itself (ring.cuh, tail.cuh).
+//
+// FP64 storage is bound by its FP64 operations (64 cycles a warp and operation; memory
+// takes 97 of a 216^3 two-field pass's 380 us): 18 a field pair and site (35 before),
+// with the Laplacian in integers (fix_lap.h), each site drifted once and shared through
+// the stage, each sum one FMA, and the potential from factors the force needs anyway.
+// The warps wait for each other's drifted plane a whole plane after writing theirs (a
+// block barrier per plane left the unit idle a fifth of the time: 457 us a pass).
+// 216^3, two fields, 5 VV4 steps and energies: 12340 us before, 10630 with a Laplacian
+// whose FP64 form for values out of range was issued predicated, 7880 with that in a
+// branch, 6590 with the deferred wait.
 #include "common.cuh"
 #include "ring.cuh"
 #include "tail.cuh"
+#include "fix_lap.h"
 
 namespace clg {
 
@@ -45,6 +56,16 @@ template <> struct ScalarPot<1> {
     d[0] = f2 * f[0];
     t[0] = T(0.25) * f2 * f2;
   }
+  // FP64: the kicked momentum (k: momentum and Laplacian part), -A3 V_{,f} added, and the
+  // potential's terms as products of two factors, w[t][0] w[t][1] x scale[t]
+  __device__ __forceinline__ static void kick64(const double (&f)[1], double A3, double, double, const double (&k)[1],
+                                                double (&pn)[1], double (&w)[1][2], double (&tot)[2]) {
+    const double f2 = f[0] * f[0];
+    pn[0] = fma(-A3, f2 * f[0], k[0]);
+    w[0][0] = w[0][1] = tot[0] = tot[1] = f2;
+  }
+  __device__ __forceinline__ static double scale(int, double) { return 0.25; }
+  static constexpr double kTotalScale = 0.25;
 };
 template <> struct ScalarPot<2> {
   static constexpr int NPOT = 2;
@@ -57,14 +78,26 @@ template <> struct ScalarPot<2> {
   template <typename T>
   __device__ __forceinline__ static void eval(const T (&f)[2], T q, T (&d)[2], T (&t)[2]) {
     const T p2 = f[0] * f[0], c2 = f[1] * f[1];
-    if constexpr (sizeof(T) == 8)
-      d[0] = f[0] * fmaT(q, c2, p2);  // phi (phi^2 + q chi^2): one operation fewer on the FP64 pipe
-    else
-      d[0] = p2 * f[0] + q * f[0] * c2;
+    d[0] = p2 * f[0] + q * f[0] * c2;
     d[1] = q * p2 * f[1];
     t[0] = T(0.25) * p2 * p2;
     t[1] = T(0.5) * q * p2 * c2;
   }
+  // V = (1/2) p2 (s - p2/2) with s = p2 + q c2, the factor of phi in the force
+  __device__ __forceinline__ static void kick64(const double (&f)[2], double A3, double q, double A3q,
+                                                const double (&k)[2], double (&pn)[2], double (&w)[2][2],
+                                                double (&tot)[2]) {
+    const double p2 = f[0] * f[0], c2 = f[1] * f[1];
+    const double s = fma(q, c2, p2);
+    pn[0] = fma(-A3, f[0] * s, k[0]);
+    pn[1] = fma(-(A3q * p2), f[1], k[1]);
+    w[0][0] = w[0][1] = w[1][0] = p2;
+    w[1][1] = c2;
+    tot[0] = p2;
+    tot[1] = fma(-0.5, p2, s);
+  }
+  __device__ __forceinline__ static double scale(int t, double q) { return t == 0 ? 0.25 : 0.5 * q; }
+  static constexpr double kTotalScale = 0.5;
 };
 
 template <typename T, int VX>
@@ -216,6 +249,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
   constexpr int VX = V16<T>::n;
   constexpr int NA = 2 * NF;
   constexpr int NPOT = ScalarPot<NF>::NPOT;
+  constexpr bool FP64 = sizeof(T) == 8;
   // RED = 1 sums: pi^2 after the kick, phi Lap phi (= -(grad^+ phi)^2 summed), V.  The pre-kick sum of
   // pi^2 is the previous kick's post-kick sum (a drift leaves pi unchanged),
   // carried in the lattice scalars.
@@ -260,6 +294,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
   Acc<T> acc[NACC];
   float nonfinite = 0.f;
   int fbuf = 0;
+  uint32_t p_drifted = 0u;  // phase of the shared planes' mbarrier (FP64)
 #pragma unroll
   for (int k = 0; k < NACC; ++k) acc[k].zero();
 
@@ -283,7 +318,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
       const long long NN = (long long)N * N;
       const int g0 = rev ? ptot - off[i + 1] : off[i];
       const T cd = rec[si.run].cf[0], A1 = rec[si.run].cf[1], A3 = rec[si.run].cf[2], q = rec[si.run].cf[3];
-      const T hq = T(0.5) * q;
+      const T hq = T(0.5) * q, A3q = A3 * q;
       const bool drifting = cd != T(0);
       T* dst[NA];
 #pragma unroll
@@ -307,10 +342,15 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
 
       // FP64 (bound by its arithmetic, not by memory): a site's drifted fields are
       // formed once and written back into its stage, where the next plane reads
-      // them as y- and x-neighbours; all threads drift the tile's two halo rows in
-      // place; then a proxy fence (bulk copies refill the stage later) and one CTA
-      // barrier per plane.  `drifting` is the same in every thread of the CTA.
-      constexpr bool SHARE = sizeof(T) == 8;
+      // them as y- and x-neighbours; the tile's two halo rows are drifted in place, by
+      // the warps without sites where these then have no more FP64 operations than the
+      // others (18 a field: 16 elements a lane), else by all; then a proxy fence (bulk
+      // copies refill the stage later) and one arrival per warp on an mbarrier, which the
+      // warps wait for one plane's kick later.  `drifting` is the same in every thread
+      // of the CTA.
+      constexpr bool SHARE = FP64;
+      const int busy = (TX * BY + 31) & ~31;  // threads of warps with sites
+      const bool idle_halo = SHARE && 16 * (THREADS - busy) >= 2 * N;
       const bool share = SHARE && drifting;
       auto share_own = [&](int s, const T (&ph)[NF][VX]) {  // active threads
         T* st = reinterpret_cast<T*>(smem + (size_t)s * P.stage_bytes_max);
@@ -320,7 +360,8 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
       auto share_halo = [&](int s) {  // every thread of the CTA
         if (!flag[0]) {
           T* st = reinterpret_cast<T*>(smem + (size_t)s * P.stage_bytes_max);
-          for (int k = tid; k < 2 * N; k += THREADS) {
+          for (int k = idle_halo ? (tid < busy ? 2 * N : tid - busy) : tid; k < 2 * N;
+               k += idle_halo ? THREADS - busy : THREADS) {
             const int e = k < N ? k : (BY + 1) * N + (k - N);
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
@@ -330,7 +371,12 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
           }
           fence_proxy_async_smem();
         }
-        __syncthreads();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(R.drifted);
+      };
+      auto share_wait = [&]() {  // the values shared last are all written
+        if (!flag[0] && !mbar_wait_bounded(R.drifted, p_drifted, P.wait_limit_ns)) flag[0] = 1;
+        p_drifted ^= 1u;
       };
 
       // drifted fields of three consecutive planes; the roles below / current /
@@ -356,12 +402,17 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
       // (the above plane is read from stage s_nxt into `above`)
       auto plane = [&](int j, const T (&below)[NF][VX], const T (&cur)[NF][VX], T (&above)[NF][VX]) {
         wait_full(s_nxt, p_nxt);
-        if (active && !flag[0]) {
-          const T* sa = stage_ptr(s_nxt);
+        if (share) share_wait();
+        const bool go = active && !flag[0];
+        if (go) read_own(stage_ptr(s_nxt), above);
+        if (share && j < nz) {
+          if (go) share_own(s_nxt, above);
+          share_halo(s_nxt);
+        }
+        if (go) {
           const T* sc = stage_ptr(s_cur);
-          read_own(sa, above);
-          if (share && j < nz) share_own(s_nxt, above);
           T lap[NF][VX], g2[VX];
+          bool in_range = true;  // FP64: the integer form holds
 #pragma unroll
           for (int v = 0; v < VX; ++v) g2[v] = T(0);
 #pragma unroll
@@ -393,68 +444,121 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
               const T xr = v == VX - 1 ? right : cur[f][v + 1];
               const T zl = below[f][v], zh = above[f][v];
               if constexpr (sizeof(T) == 8) {
-                // FP64: the six neighbours summed, then -6 c in one FMA (the fewest
-                // operations on the narrow FP64 pipe); FP32 keeps each direction's
-                // small difference from its own pair sum
-                lap[f][v] = fmaT(T(-6), c, ((xl + xr) + (yl[v] + yh[v])) + (zl + zh));
+                bool ok;
+                lap[f][v] = fix_lap(fix_val(xl), fix_val(xr), fix_val(yl[v]), fix_val(yh[v]), fix_val(zl), fix_val(zh),
+                                    fix_val(c), &ok);
+                in_range = in_range && ok;
               } else {
+                // FP32 keeps each direction's small difference from its own pair sum
                 lap[f][v] = ((xl + xr) - T(2) * c) + ((yl[v] + yh[v]) - T(2) * c) +
                             ((zl + zh) - T(2) * c);
               }
               if (RED == 2) {  // forward differences (eq. EK_EG_EV with grad^+)
                 const T zp = dir > 0 ? zh : zl;
                 const T gx = xr - c, gy = yh[v] - c, gz = zp - c;
-                gf += gx * gx + gy * gy + gz * gz;
+                if constexpr (FP64)
+                  acc[6 * f + 2].s = fma(gz, gz, fma(gy, gy, fma(gx, gx, acc[6 * f + 2].s)));
+                else
+                  gf += gx * gx + gy * gy + gz * gz;
               } else if (RED == 1) {
                 // sum_n (grad^+ phi)^2 = -sum_n phi Lap phi (summation by parts on the
                 // periodic lattice): one FMA on the Laplacian the kick needs anyway
-                g2[v] = fmaT(c, lap[f][v], g2[v]);
+                if constexpr (!FP64) g2[v] = fmaT(c, lap[f][v], g2[v]);
               }
             }
-            if (RED == 2) acc[6 * f + 2].add(gf);
+            if constexpr (RED == 2 && !FP64) acc[6 * f + 2].add(gf);
+          }
+          if constexpr (FP64) {
+            // the thread's sites again, in FP64 (one block of all of them: a branch, where a
+            // short one would be issued predicated and take its time on the FP64 unit)
+            if (!in_range) {
+#pragma unroll
+              for (int f = 0; f < NF; ++f) {
+                const T* ph = sc + (size_t)(2 * f) * arr_elems;
+                T yl[VX], yh[VX];
+                ld_vec<T, VX>(yl, ph + ty * N + x0);
+                ld_vec<T, VX>(yh, ph + (ty + 2) * N + x0);
+#pragma unroll
+                for (int v = 0; v < VX; ++v)
+                  lap[f][v] = fp64_lap(v == 0 ? ph[exl] : cur[f][v - 1], v == VX - 1 ? ph[exr] : cur[f][v + 1], yl[v],
+                                       yh[v], below[f][v], above[f][v], cur[f][v]);
+              }
+            }
           }
           T pn[NF][VX], pic[NF][VX];  // momenta of the current plane, from its stage
 #pragma unroll
           for (int f = 0; f < NF; ++f) ld_vec<T, VX>(pic[f], sc + (size_t)(2 * f + 1) * arr_elems + own);
-          T spost = T(0), vs = T(0), gsum = T(0);
+          if constexpr (FP64) {
+            // every sum one FMA into its accumulator (FP32 adds a plane's terms first)
 #pragma unroll
-          for (int v = 0; v < VX; ++v) {
-            T fv[NF], dv[NF], tv[NPOT];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) fv[f] = cur[f][v];
-            ScalarPot<NF>::eval(fv, q, dv, tv);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              // FP32 adds the small increment last (one rounding at the momentum's
-              // size); FP64 takes two FMAs
-              if constexpr (sizeof(T) == 8)
-                pn[f][v] = fmaT(-A3, dv[f], fmaT(A1, lap[f][v], pic[f][v]));
-              else
-                pn[f][v] = pic[f][v] + (A1 * lap[f][v] - A3 * dv[f]);
-            }
-            if (RED == 1) {
-#pragma unroll
-              for (int f = 0; f < NF; ++f) spost = fmaT(pn[f][v], pn[f][v], spost);
-              vs += ScalarPot<NF>::total(fv, hq);
-              gsum += g2[v];
-            } else if (RED == 2) {
+            for (int v = 0; v < VX; ++v) {
+              double fv[NF], k[NF], p[NF], w[NPOT][2], tot[2];
 #pragma unroll
               for (int f = 0; f < NF; ++f) {
-                acc[6 * f + 0].add(pic[f][v] * pic[f][v]);
-                acc[6 * f + 1].add(pn[f][v] * pn[f][v]);
-                acc[6 * f + 3].add(fv[f]);
-                acc[6 * f + 4].add(fv[f] * fv[f]);
-                acc[6 * f + 5].add(pn[f][v]);
-                if (!isfinite(pn[f][v])) nonfinite += 1.f;
+                fv[f] = cur[f][v];
+                k[f] = fma(A1, lap[f][v], pic[f][v]);
               }
+              ScalarPot<NF>::kick64(fv, A3, q, A3q, k, p, w, tot);
 #pragma unroll
-              for (int t = 0; t < NPOT; ++t) acc[6 * NF + t].add(tv[t]);
+              for (int f = 0; f < NF; ++f) {
+                pn[f][v] = p[f];
+                if constexpr (RED == 1) {
+                  acc[0].s = fma(p[f], p[f], acc[0].s);
+                  acc[1].s = fma(fv[f], lap[f][v], acc[1].s);
+                }
+                if constexpr (RED == 2) {
+                  acc[6 * f + 0].s = fma(pic[f][v], pic[f][v], acc[6 * f + 0].s);
+                  acc[6 * f + 1].s = fma(p[f], p[f], acc[6 * f + 1].s);
+                  acc[6 * f + 3].s += fv[f];
+                  acc[6 * f + 4].s = fma(fv[f], fv[f], acc[6 * f + 4].s);
+                  acc[6 * f + 5].s += p[f];
+                  // (an FP64 comparison would be one more operation on that unit)
+                  if ((__double2hiint(p[f]) & 0x7ff00000) == 0x7ff00000) nonfinite += 1.f;
+                }
+              }
+              if constexpr (RED == 1) acc[2].s = fma(tot[0], tot[1], acc[2].s);
+              if constexpr (RED == 2) {
+#pragma unroll
+                for (int t = 0; t < NPOT; ++t) acc[6 * NF + t].s = fma(w[t][0], w[t][1], acc[6 * NF + t].s);
+              }
             }
-          }
-          if (RED == 1) {
-            acc[0].add(spost);
-            acc[1].add(gsum);
-            acc[2].add(vs);
+          } else {
+            T spost = T(0), vs = T(0), gsum = T(0);
+#pragma unroll
+            for (int v = 0; v < VX; ++v) {
+              T fv[NF], dv[NF], tv[NPOT];
+#pragma unroll
+              for (int f = 0; f < NF; ++f) fv[f] = cur[f][v];
+              ScalarPot<NF>::eval(fv, q, dv, tv);
+#pragma unroll
+              for (int f = 0; f < NF; ++f) {
+                // the small increment last: one rounding at the momentum's size
+                pn[f][v] = pic[f][v] + (A1 * lap[f][v] - A3 * dv[f]);
+              }
+              if (RED == 1) {
+#pragma unroll
+                for (int f = 0; f < NF; ++f) spost = fmaT(pn[f][v], pn[f][v], spost);
+                vs += ScalarPot<NF>::total(fv, hq);
+                gsum += g2[v];
+              } else if (RED == 2) {
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                  acc[6 * f + 0].add(pic[f][v] * pic[f][v]);
+                  acc[6 * f + 1].add(pn[f][v] * pn[f][v]);
+                  acc[6 * f + 3].add(fv[f]);
+                  acc[6 * f + 4].add(fv[f] * fv[f]);
+                  acc[6 * f + 5].add(pn[f][v]);
+                  if (!isfinite(pn[f][v])) nonfinite += 1.f;
+                }
+#pragma unroll
+                for (int t = 0; t < NPOT; ++t) acc[6 * NF + t].add(tv[t]);
+              }
+            }
+            if (RED == 1) {
+              acc[0].add(spost);
+              acc[1].add(gsum);
+              acc[2].add(vs);
+            }
           }
           if (P.write) {
             const long long gi = (long long)seg_plane_z(z0, nz, N, dir, j) * NN + (long long)y * N + x0;
@@ -465,7 +569,6 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
             }
           }
         }
-        if (share && j < nz) share_halo(s_nxt);
         release(g0 + j, s_cur);
         s_cur = s_nxt;
         p_cur = p_nxt;
@@ -483,6 +586,13 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_scalar(const __grid_consta
 
       if (!run_end) continue;
 
+      if constexpr (FP64) {  // the potential's sums were kept without their constant factors
+        if constexpr (RED == 1) acc[2].s *= ScalarPot<NF>::kTotalScale;
+        if constexpr (RED == 2) {
+#pragma unroll
+          for (int t = 0; t < NPOT; ++t) acc[6 * NF + t].s *= ScalarPot<NF>::scale(t, q);
+        }
+      }
       double* rb = R.red + fbuf * CONSUMER_WARPS * NQ;
       fbuf ^= 1;
       if (!ring_flush<NACC, NUSED>(R, P, si, pass, acc, nonfinite, rb, (TX * BY + 31) >> 5, warp, lane)) goto timeout;

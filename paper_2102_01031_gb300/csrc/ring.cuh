@@ -44,6 +44,7 @@ struct Ring {
   unsigned char* stages;  // S stages of stage_bytes
   uint64_t* full;         // one mbarrier per stage: all copies of the stage landed
   unsigned* released;     // warps done with each stage
+  uint64_t* drifted;      // mbarrier, one arrival per warp (FP64 scalar pass)
   int* off;               // first plane of each segment, and the total
   double* red;            // [33][NQ] reduction scratch
   volatile int* flag;     // [0] timed out, [1] runs of the CTA, [2] lattice of the last run, [3] #pending tails
@@ -62,6 +63,7 @@ __device__ __forceinline__ Ring ring_view(unsigned char* smem, const PassArgs& P
   unsigned char* tail = smem + (size_t)R.S * R.stage_bytes;
   R.full = reinterpret_cast<uint64_t*>(tail + SM_FULL);
   R.released = reinterpret_cast<unsigned*>(tail + SM_RELEASED);
+  R.drifted = reinterpret_cast<uint64_t*>(tail + SM_DRIFTED);
   R.off = reinterpret_cast<int*>(tail + SM_OFF);
   R.red = reinterpret_cast<double*>(tail + SM_RED);
   R.flag = reinterpret_cast<volatile int*>(tail + SM_FLAG);
@@ -79,6 +81,7 @@ __device__ void ring_setup(const Ring& R, const PassArgs& P, int sb, int ns) {
     mbar_init(&R.full[s], 1);
     R.released[s] = 0u;
   }
+  mbar_init(R.drifted, CONSUMER_WARPS);
   fence_mbar_init();
   R.flag[0] = 0;
   R.flag[2] = ns > 0 ? P.segs[sb].lat : 0;
