@@ -78,17 +78,11 @@ __global__ void __launch_bounds__(256, (RED == 2 || sizeof(T) == 8) ? 1 : 2) dk_
   constexpr size_t slot_b = su2_slot_bytes(TX, TY, sizeof(T), FULL);
 
   // the deferred drift and the kick's coefficients
-  T drift[3];
-  if (lane == 0) {
-    const double cdA64 = __ldcg(&P.sc->cdA);
-    drift[0] = (T)__ldcg(&P.sc->cd);
-    drift[1] = (T)cdA64;
-    drift[2] = (T)(0.5 * L.gQB * L.dx * cdA64);  // half the SU(2) drift angle per momentum
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) drift[k] = __shfl_sync(0xffffffffu, drift[k], 0);
-  const T cd = drift[0], cdA = drift[1], hB = drift[2];
-  const Su2Coef<T> cf = su2_coefficients<T>(L, P.sc, P.ck, lane);
+  __shared__ Su2Pass<T> coef_s;
+  if (warp == 0) su2_coefficients<T>(L, P.sc, P.ck, __ldcg(&P.sc->cd), __ldcg(&P.sc->cdA), lane, &coef_s);
+  __syncthreads();
+  const T cd = coef_s.cd, cdA = coef_s.cdA, hB = coef_s.hB;
+  const Su2Coef<T> cf = coef_s.k;
   const bool drifting = cd != T(0) || cdA != T(0);
 
   Acc<T> acc[NACC];

@@ -132,20 +132,14 @@ __global__ void __launch_bounds__(TX * TY, (RED == 2 || sizeof(T) == 8) ? 1 : 20
   const int ntx = N / TX, ntiles = ntx * (N / TY), nzc = L.su2_nzc, nitems = ntiles * nzc;
 
   // this pass's drift, after its kick, and the kick's coefficients
-  T drift[3];
-  if (lane == 0) {
+  __shared__ Su2Pass<T> coef_s;
+  if (warp == NW - 1) {
     double kd64, kdA64;
     ScalarState W;
     load_state_cg(W, P.sc);
     kd_drift_coefficients(L, W, P.dnext, kd64, kdA64);
-    drift[0] = (T)kd64;
-    drift[1] = (T)kdA64;
-    drift[2] = (T)(0.5 * L.gQB * L.dx * kdA64);  // half the SU(2) drift angle per momentum
+    su2_coefficients<T>(L, P.sc, P.ck, kd64, kdA64, lane, &coef_s);
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) drift[k] = __shfl_sync(0xffffffffu, drift[k], 0);
-  const T kd = drift[0], kdA = drift[1], hB = drift[2];
-  const Su2Coef<T> cf = su2_coefficients<T>(L, P.sc, P.ck, lane);
 
   if (tid == 0) {
     for (int s = 0; s < 3; ++s) {
@@ -156,6 +150,8 @@ __global__ void __launch_bounds__(TX * TY, (RED == 2 || sizeof(T) == 8) ? 1 : 20
     tflag = 0;
   }
   __syncthreads();
+  const T kd = coef_s.cd, kdA = coef_s.cdA, hB = coef_s.hB;
+  const Su2Coef<T> cf = coef_s.k;
 
   // The CTA's planes form one sequence of positions (item by item, each item's
   // planes z0 - 1 .. z0 + nz); position p lives in stage p mod 3.  produced: the

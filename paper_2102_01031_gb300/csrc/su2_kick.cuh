@@ -122,35 +122,52 @@ __device__ __forceinline__ P3 qvec2_cb(const Q2& a, const Q2& b) {
 
 // Coefficients of a pass in the storage precision: kicks (doublet Laplacian, potential,
 // U(1) current and curl, SU(2) current and plaquettes, vphi's current), phases per A_i,
-// potential constants; FP64 products by one lane of each warp, broadcast.
+// potential constants.
 template <typename T>
 struct Su2Coef {
   T A1, A3, AJA, ACA, AJB, AMB, gd, v2, lam, lam2, qG, qH, gdc, AJC;
 };
+// A pass's coefficients in shared memory, and its drift: of the fields, of the links, and
+// half the SU(2) links' drift angle per momentum.
 template <typename T>
-__device__ __forceinline__ Su2Coef<T> su2_coefficients(const LatConst& L, const LatScalars* SC, double ck, int lane) {
-  T cf[14];
-  if (lane == 0) {
-    const double ap1 = __ldcg(&SC->apow1), apm1 = __ldcg(&SC->apowm1), dx = L.dx;
-    cf[0] = (T)(ck * ap1 * L.inv_dx2);
-    cf[1] = (T)(ck * __ldcg(&SC->apow3));
-    cf[2] = (T)(ck * ap1 * L.fo2 * L.gQ / dx);
-    cf[3] = (T)(L.gQ != 0.0 ? -ck * apm1 / (L.gQ * dx * dx * dx) : 0.0);
-    cf[4] = (T)(ck * ap1 * L.fo2 * L.gQB / (2.0 * dx));
-    cf[5] = (T)(-2.0 * ck * apm1 / (L.gQB * dx * dx * dx));
-    cf[6] = (T)(L.gQ * dx);
-    cf[7] = (T)(L.v * L.v);
-    cf[8] = (T)L.lam;
-    cf[9] = (T)(2.0 * L.lam);
-    cf[10] = (T)L.qG;
-    cf[11] = (T)L.qH;
-    cf[12] = (T)(L.Qc * L.gQ * dx);
-    cf[13] = (T)(ck * ap1 * L.fo2 * L.Qc * L.gQ / dx);
+struct Su2Pass {
+  Su2Coef<T> k;
+  T cd, cdA, hB;
+};
+// By one whole warp: lane l forms value l as a product of up to five numbers over a product
+// of up to four (in every warp of a CTA and one value after the other they were 89 FP64
+// operations a thread, 12 of the 165 us of a 128^3 pass without sums).
+template <typename T>
+__device__ __noinline__ void su2_coefficients(const LatConst& L, const LatScalars* SC, double ck, double cd,
+                                              double cdA, int lane, Su2Pass<T>* out) {
+  static_assert(sizeof(Su2Pass<T>) == 17 * sizeof(T), "the values by lane");
+  const double ap1 = __ldcg(&SC->apow1), apm1 = __ldcg(&SC->apowm1), ap3 = __ldcg(&SC->apow3);
+  const double dx = L.dx, gQ = L.gQ, gQB = L.gQB;
+  double n0 = 1.0, n1 = 1.0, n2 = 1.0, n3 = 1.0, n4 = 1.0, d0 = 1.0, d1 = 1.0, d2 = 1.0, d3 = 1.0;
+  switch (lane) {
+    case 0: n0 = ck; n1 = ap1; n2 = L.inv_dx2; break;
+    case 1: n0 = ck; n1 = ap3; break;
+    case 2: n0 = ck; n1 = ap1; n2 = L.fo2; n3 = gQ; d0 = dx; break;
+    case 3: n0 = -ck; n1 = apm1; d0 = gQ; d1 = d2 = d3 = dx; break;
+    case 4: n0 = ck; n1 = ap1; n2 = L.fo2; n3 = gQB; d0 = 2.0; d1 = dx; break;
+    case 5: n0 = -2.0; n1 = ck; n2 = apm1; d0 = gQB; d1 = d2 = d3 = dx; break;
+    case 6: n0 = gQ; n1 = dx; break;
+    case 7: n0 = n1 = L.v; break;
+    case 8: n0 = L.lam; break;
+    case 9: n0 = 2.0; n1 = L.lam; break;
+    case 10: n0 = L.qG; break;
+    case 11: n0 = L.qH; break;
+    case 12: n0 = L.Qc; n1 = gQ; n2 = dx; break;
+    case 13: n0 = ck; n1 = ap1; n2 = L.fo2; n3 = L.Qc; n4 = gQ; d0 = dx; break;
+    case 14: n0 = cd; break;
+    case 15: n0 = cdA; break;
+    case 16: n0 = 0.5; n1 = gQB; n2 = dx; n3 = cdA; break;
+    default: break;
   }
-#pragma unroll
-  for (int k = 0; k < 14; ++k) cf[k] = __shfl_sync(0xffffffffu, cf[k], 0);
-  return Su2Coef<T>{cf[0], cf[1], cf[2], cf[3],  cf[4],  cf[5],  cf[6],
-                    cf[7], cf[8], cf[9], cf[10], cf[11], cf[12], cf[13]};
+  const double num = n0 * n1 * n2 * n3 * n4, den = d0 * d1 * d2 * d3;
+  // without a U(1) charge the links' plaquettes do not act (value 3)
+  const double v = lane == 3 && gQ == 0.0 ? 0.0 : num / den;
+  if (lane < 17) reinterpret_cast<T*>(out)[lane] = (T)v;
 }
 
 // Carried along z from the plane below: U(1) plaquette sines xz and yz at n - z, the lower
