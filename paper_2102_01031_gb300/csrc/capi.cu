@@ -54,7 +54,7 @@ cudaError_t launch_ic_assemble(int, void*, void*, const double2*, const double2*
                                const LatScalars*, double, double, long long, cudaStream_t);
 cudaError_t launch_fft_axis(double2*, const FftPlan&, cudaStream_t);
 cudaError_t launch_fft_twiddles(int4*, int, int, cudaStream_t);
-cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftPlan& pl, double dk, int nb,
+cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftPlan& pl, int nb,
                                  int nblk, double* part, double kIR, double dx, double* out, cudaStream_t st,
                                  const int* bin_of, const double* geo);
 cudaError_t launch_shell_geometry(int N, double dk, int nb, int nblk, int* bin_of, double* geo, double* part,
@@ -1563,7 +1563,7 @@ cl_status cl_ensemble_spectrum(cl_ctx* c, const int* lats, int nl, int field, in
   }
   for (int i = 0; i < nl; ++i) {
     const int l = lats[i];
-    CU(launch_real_spectrum(c->fp32, arr_ptr(c, l, c->parity, a), F, pl, dk_bin, nb, nblk, part, H.kIR, H.dx,
+    CU(launch_real_spectrum(c->fp32, arr_ptr(c, l, c->parity, a), F, pl, nb, nblk, part, H.kIR, H.dx,
                             bins + (size_t)i * 3 * nb, c->stream, c->d_bin_of, c->d_geo));
     c->launches += 5;
   }

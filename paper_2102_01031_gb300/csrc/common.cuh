@@ -202,6 +202,9 @@ struct FftPlan {
   int nu;                // lines along the fastest other index (axes 1, 2: the columns kept, <= pitch)
   int ng;                // groups of `batch` lines among them
   FastDiv dN, dB, dH, dg;  // N, batch, N/2 + 1, ng
+  const int* ein;        // exponents of the lines that an array in fixed point comes from (fft_lines_kernel)
+  int* eout;             // and of those it goes to
+  double* pout;          // where the last axis of a spectrum leaves |F|^2
 };
 
 // ---------------------------------------------------------------------------

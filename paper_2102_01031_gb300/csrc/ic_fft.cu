@@ -15,6 +15,8 @@
 
 #include <algorithm>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "fix_fft.h"
 
@@ -432,7 +434,14 @@ constexpr int FFT_HELD = 4;  // elements a thread holds between its load and the
 // axis 0: j + P (u + N w) (rows, P = N); axis 1: u + P (j + N w); axis 2: u + P (w + N j).
 // A CTA takes `batch` lines with consecutive u (and one w); lines with u >= nu are
 // not loaded or stored (the last group of a half spectrum's N/2 + 1 columns).
-template <int NC>
+// IO: what the array holds before and after: FFT_FP64 FP64 values; FFT_FIX_FIX fixed point with an
+// exponent per line of the axis before (rows in pairs, axis 1 only) and per line of this one;
+// FFT_FIX_POWER the former (axis 2), then |F|^2 in FP64 in an array of its own (half the
+// bytes, and its two FP64 operations run beside the integer ones, which bound this kernel;
+// the shell sums were bound by theirs).  256^3 from an FP32 field: rows 185 -> 170 us, y
+// 166 -> 151, z with the squares 166 -> 174, shell sums 100 -> 67.
+constexpr int FFT_FP64 = 0, FFT_FIX_FIX = 1, FFT_FIX_POWER = 2;
+template <int NC, int IO>
 __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const __grid_constant__ FftPlan plan) {
   extern __shared__ __align__(16) unsigned char fbuf[];
   const int N = NC ? NC : plan.N, B = NC ? fft_batch_of(NC) : plan.batch, Pt = N + 1;
@@ -459,22 +468,34 @@ __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const 
   };
   // load (the host picks nt so that a thread holds at most FFT_HELD elements), the
   // lines' exponents and sums, fixed point
-  double2 h[FFT_HELD];
+  typedef typename std::conditional<IO == FFT_FP64, double2, CFix>::type Elem;
+  Elem h[FFT_HELD];
   int hl[FFT_HELD];  // line; -1: nothing
+  int hq[FFT_HELD];  // fixed point: the exponent
 #pragma unroll
   for (int i = 0; i < FFT_HELD; ++i) {
     const int t = tid + i * nt;
     int l = 0, p = 0;
     const long long at = t < B * N ? place(t, l, p) : -1;
-    h[i] = at >= 0 ? data[at] : make_double2(0.0, 0.0);
+    h[i] = Elem{};
+    hq[i] = 0;
     hl[i] = at >= 0 ? l : -1;
+    if (at >= 0) {
+      h[i] = reinterpret_cast<const Elem*>(data)[at];
+      if constexpr (IO == FFT_FIX_FIX) hq[i] = __ldg(plan.ein + ((w0 * N + p) >> 1));
+      if constexpr (IO == FFT_FIX_POWER) hq[i] = __ldg(plan.ein + p * P + (int)u0 + l);
+    }
   }
   // a thread's elements all lie on its first one's line where the block is a multiple of
   // the batch (columns): one update of the line's words instead of FFT_HELD
   const bool one = !rows && plan.dB.mod(nt, plan.dB.div(nt)) == 0;
   int top[FFT_HELD];
 #pragma unroll
-  for (int i = 0; i < FFT_HELD; ++i) top[i] = max(top_of(h[i].x), top_of(h[i].y));
+  for (int i = 0; i < FFT_HELD; ++i) {
+    if constexpr (IO == FFT_FP64) top[i] = max(top_of(h[i].x), top_of(h[i].y));
+    else top[i] = fix_top(h[i], hq[i]);
+    if (hq[i] == FIX_NAN) hq[i] = 0;
+  }
   if (one) {
     line_reduce<true>(M.top, hl[0], max(max(top[0], top[1]), max(top[2], top[3])));
   } else {
@@ -485,8 +506,14 @@ __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const 
   int sum[FFT_HELD];
 #pragma unroll
   for (int i = 0; i < FFT_HELD; ++i) {
-    const int E = expo_of<double>(hl[i] >= 0 ? M.top[hl[i]] : 0);
-    sum[i] = hl[i] >= 0 ? size_of(h[i].x, E) + size_of(h[i].y, E) : 0;
+    const int line_top = hl[i] >= 0 ? M.top[hl[i]] : 0;
+    if constexpr (IO == FFT_FP64) {
+      const int E = expo_of<double>(line_top);
+      sum[i] = size_of(h[i].x, E) + size_of(h[i].y, E);
+    } else {
+      sum[i] = fix_units(h[i].x, hq[i], line_top) + fix_units(h[i].y, hq[i], line_top);
+    }
+    if (hl[i] < 0) sum[i] = 0;
   }
   if (one) {
     line_reduce<false>(M.sum, hl[0], (sum[0] + sum[1]) + (sum[2] + sum[3]));
@@ -495,8 +522,14 @@ __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const 
     for (int i = 0; i < FFT_HELD; ++i) line_reduce<false>(M.sum, hl[i], sum[i]);
   }
   __syncthreads();
-  for (int l = tid; l < B; l += nt) M.sc[l] = line_scale<double>(expo_of<double>(M.top[l]), M.sum[l]);
+  for (int l = tid; l < B; l += nt) {
+    if constexpr (IO == FFT_FP64) M.sc[l] = line_scale<double>(expo_of<double>(M.top[l]), M.sum[l]);
+    else M.sc[l].E = fix_line_exponent(M.top[l], M.sum[l]);
+  }
   __syncthreads();
+  if constexpr (IO == FFT_FIX_FIX)
+    for (int l = tid; l < B; l += nt)
+      if (u0 + l < nu) plan.eout[(long long)w0 * P + u0 + l] = M.sc[l].E;
 #pragma unroll
   for (int i = 0; i < FFT_HELD; ++i) {
     const int t = tid + i * nt;
@@ -504,7 +537,11 @@ __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const 
       int l = 0, p = 0;
       place(t, l, p);
       const LineScale sc = M.sc[l];
-      M.a[l * Pt + p] = CFix{to_fix(h[i].x, sc), to_fix(h[i].y, sc)};
+      if constexpr (IO == FFT_FP64) M.a[l * Pt + p] = CFix{to_fix(h[i].x, sc), to_fix(h[i].y, sc)};
+      else {
+        const int to = sc.E == FIX_NAN ? hq[i] : sc.E;
+        M.a[l * Pt + p] = CFix{fix_rescale(h[i].x, hq[i], to), fix_rescale(h[i].y, hq[i], to)};
+      }
     }
   }
   __syncthreads();
@@ -516,11 +553,18 @@ __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const 
     const long long at = place(t, l, p);
     if (at < 0) continue;
     const LineScale sc = M.sc[l];
-    const int q = sc.E - FixIO<double>::BIAS - sc.up;
     const CFix v = a[l * Pt + p];
-    data[at] = sc.E == FixIO<double>::ETOP
-                   ? make_double2(fix_nan(), fix_nan())
-                   : make_double2(from_fix(v.x, q, sc.plain), from_fix(v.y, q, sc.plain));
+    if constexpr (IO == FFT_FIX_FIX) {
+      reinterpret_cast<CFix*>(data)[at] = v;
+    } else {
+      const bool nan = sc.E == (IO == FFT_FP64 ? FixIO<double>::ETOP : FIX_NAN);
+      const int q = IO == FFT_FP64 ? sc.E - FixIO<double>::BIAS - sc.up : sc.E;
+      const bool plain = IO == FFT_FP64 ? sc.plain : q > -1000 && q < 900;
+      const double2 f = nan ? make_double2(fix_nan(), fix_nan())
+                            : make_double2(from_fix(v.x, q, plain), from_fix(v.y, q, plain));
+      if constexpr (IO == FFT_FP64) data[at] = f;
+      else plan.pout[at] = fma(f.x, f.x, f.y * f.y);
+    }
   }
 }
 
@@ -531,7 +575,7 @@ __global__ void __launch_bounds__(512, 2) fft_lines_kernel(double2* data, const 
 // of real transforms: X_a(k) = (Z(k) + Z^*(N-k))/2, X_b(k) = (Z(k) - Z^*(N-k))/(2i),
 // for k = 0 .. N/2.  A CTA takes `batch` row pairs.
 template <typename T, int NC>
-__global__ void __launch_bounds__(512, 2) rfft_rows_kernel(const T* f, double2* H, const __grid_constant__ FftPlan plan) {
+__global__ void __launch_bounds__(512, 2) rfft_rows_kernel(const T* f, CFix* H, const __grid_constant__ FftPlan plan) {
   extern __shared__ __align__(16) unsigned char fbuf[];
   const int N = NC ? NC : plan.N, B = NC ? fft_batch_of(NC) : plan.batch, Pt = N + 1, NH = N / 2 + 1;
   const int nt = blockDim.x, tid = threadIdx.x;
@@ -576,71 +620,15 @@ __global__ void __launch_bounds__(512, 2) rfft_rows_kernel(const T* f, double2* 
   for (int t = tid; t < B * NH; t += nt) {
     const int l = NC ? t / NH : plan.dH.div(t), k = t - l * NH;
     const CFix Z = a[l * Pt + k], Y = a[l * Pt + (k == 0 ? 0 : N - k)];  // Y = Z(N - k)
-    const LineScale sc = M.sc[l];
-    const int q = sc.E - FixIO<T>::BIAS - sc.up - 1;  // with the halves
-    // the sums are twice a row's transform, below 2^63
-    double2 Xa = make_double2(from_fix(Z.x + Y.x, q, sc.plain), from_fix(Z.y - Y.y, q, sc.plain));
-    double2 Xb = make_double2(from_fix(Z.y + Y.y, q, sc.plain), from_fix(Y.x - Z.x, q, sc.plain));
-    if (sc.E == FixIO<T>::ETOP) Xa.x = Xa.y = Xb.x = Xb.y = fix_nan();
+    // twice a row's transform, below 2^63; the halves go into the exponent
     const long long ra = 2 * (p0 + l);
-    H[ra * NH + k] = Xa;
-    H[(ra + 1) * NH + k] = Xb;
-  }
-}
-
-// Shell sums of a half spectrum H (as rfft_rows_kernel writes it, all three
-// axes transformed): each kept mode stands for itself and, for 0 < kx < N/2,
-// for its conjugate partner (-kx, -ky, -kz) with the same |F|^2 and |n|, so it
-// counts twice.  Runs of equal bins along kx are summed before the atomics.
-__global__ void bin_half_kernel(const double2* H, int N, double dk, int nb, double* part) {
-  extern __shared__ double sb[];
-  double* sp = sb;
-  double* sn = sb + nb;
-  double* sc = sb + 2 * nb;
-  for (int i = threadIdx.x; i < 3 * nb; i += blockDim.x) sb[i] = 0.0;
-  __syncthreads();
-  constexpr int CH = 8;
-  const int NH = N / 2 + 1, nchr = (NH + CH - 1) / CH;
-  const long long nch = (long long)N * N * nchr;
-  for (long long ch = (long long)blockIdx.x * blockDim.x + threadIdx.x; ch < nch;
-       ch += (long long)gridDim.x * blockDim.x) {
-    const long long row = ch / nchr;
-    const int x0 = (int)(ch % nchr) * CH;
-    const int y = (int)(row % N), z = (int)(row / N);
-    const int ny = y <= N / 2 ? y : y - N, nz = z <= N / 2 ? z : z - N;
-    const int c2 = ny * ny + nz * nz;
-    int cur = -1;
-    double rp = 0.0, rn = 0.0, rc = 0.0;
-    const int x1 = x0 + CH < NH ? x0 + CH : NH;
-    for (int kx = x0; kx < x1; ++kx) {
-      const int m2 = kx * kx + c2;
-      if (m2 == 0) continue;  // the zero mode is in no bin
-      const double nn = sqrt((double)m2);
-      int bb = (int)floor(nn / dk);
-      if (bb >= nb) bb = nb - 1;
-      if (bb != cur) {
-        if (cur >= 0) {
-          atomicAdd(&sp[cur], rp);
-          atomicAdd(&sn[cur], rn);
-          atomicAdd(&sc[cur], rc);
-        }
-        cur = bb;
-        rp = rn = rc = 0.0;
-      }
-      const double wgt = (kx == 0 || kx == N / 2) ? 1.0 : 2.0;
-      const double2 v = H[row * NH + kx];
-      rp += wgt * (v.x * v.x + v.y * v.y);
-      rn += wgt * nn;
-      rc += wgt;
-    }
-    if (cur >= 0) {
-      atomicAdd(&sp[cur], rp);
-      atomicAdd(&sn[cur], rn);
-      atomicAdd(&sc[cur], rc);
+    H[ra * NH + k] = CFix{Z.x + Y.x, Z.y - Y.y};
+    H[(ra + 1) * NH + k] = CFix{Z.y + Y.y, Y.x - Z.x};
+    if (k == 0) {
+      const LineScale sc = M.sc[l];
+      plan.eout[p0 + l] = sc.E == FixIO<T>::ETOP ? FIX_NAN : sc.E - FixIO<T>::BIAS - sc.up - 1;
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 3 * nb; i += blockDim.x) part[(size_t)blockIdx.x * 3 * nb + i] = sb[i];
 }
 
 template <typename T>
@@ -844,8 +832,9 @@ __global__ void geo_final_kernel(const double* part, int nblk, int nb, double* g
 
 // Shell sums of |F|^2 of a half spectrum with the cached bins: each kept mode
 // counts twice for 0 < kx < N/2 (its conjugate partner), runs of equal bins
-// along kx are summed before the atomic.  Partial rows of nb per block.
-__global__ void bin_power_half_kernel(const double2* H, const int* bin_of, int N, int nb, int nc, double* part) {
+// along kx are summed before the atomic.  Partial rows of nb per block.  Half of each
+// mode's share is added up, the two edge columns' halved, all doubled at the end.
+__global__ void bin_power_half_kernel(const double* H, const int* bin_of, int N, int nb, int nc, double* part) {
   extern __shared__ double sb_all[];
   for (int i = threadIdx.x; i < nc * nb; i += blockDim.x) sb_all[i] = 0.0;
   // nc copies of the bins, a warp adds to one of them: an FP64 addition to shared memory is
@@ -862,36 +851,35 @@ __global__ void bin_power_half_kernel(const double2* H, const int* bin_of, int N
     const int y = (int)(row % N), z = (int)(row / N);
     const int ny = y <= N / 2 ? y : y - N, nz = z <= N / 2 ? z : z - N;
     const int c2 = ny * ny + nz * nz;
-    // runs of equal bins, two FP64 operations per mode; the columns between 0 and N/2
-    // stand for their partners too, the two edge columns are added once, apart
     int cur = -1;
     double rp = 0.0;
-    double2 v[CH];
+    double v[CH];
 #pragma unroll
-    for (int i = 0; i < CH; ++i) v[i] = x0 + i < NH ? H[row * NH + x0 + i] : make_double2(0.0, 0.0);
+    for (int i = 0; i < CH; ++i) v[i] = x0 + i < NH ? H[row * NH + x0 + i] : 0.0;
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
       const int kx = x0 + i;
       if (kx >= NH) break;
       const int b = bin_of[kx * kx + c2];
       if (kx == 0 || kx == N / 2) {
-        if (b >= 0) atomicAdd(&sb[b], fma(v[i].x, v[i].x, v[i].y * v[i].y));
+        if (b >= 0) atomicAdd(&sb[b], 0.5 * v[i]);
         continue;
       }
       if (b != cur) {
-        if (cur >= 0) atomicAdd(&sb[cur], 2.0 * rp);
+        if (cur >= 0) atomicAdd(&sb[cur], rp);
         cur = b;
-        rp = 0.0;
+        rp = v[i];
+      } else {
+        rp += v[i];
       }
-      rp = fma(v[i].x, v[i].x, fma(v[i].y, v[i].y, rp));
     }
-    if (cur >= 0) atomicAdd(&sb[cur], 2.0 * rp);
+    if (cur >= 0) atomicAdd(&sb[cur], rp);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < nb; i += blockDim.x) {
     double t = 0.0;
     for (int c = 0; c < nc; ++c) t += sb_all[c * nb + i];
-    part[(size_t)blockIdx.x * nb + i] = t;
+    part[(size_t)blockIdx.x * nb + i] = 2.0 * t;
   }
 }
 
@@ -1035,11 +1023,12 @@ cudaError_t launch_fft_twiddles(int4* tw, int N, int sign, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_fft_axis(double2* data, const FftPlan& pl, cudaStream_t st) {
-  void (*kern)(double2*, const FftPlan) = pl.N == 128   ? fft_lines_kernel<128>
-                                          : pl.N == 256 ? fft_lines_kernel<256>
-                                          : pl.N == 512 ? fft_lines_kernel<512>
-                                                        : fft_lines_kernel<0>;
+template <int IO>
+static cudaError_t launch_lines(double2* data, const FftPlan& pl, cudaStream_t st) {
+  void (*kern)(double2*, const FftPlan) = pl.N == 128   ? fft_lines_kernel<128, IO>
+                                          : pl.N == 256 ? fft_lines_kernel<256, IO>
+                                          : pl.N == 512 ? fft_lines_kernel<512, IO>
+                                                        : fft_lines_kernel<0, IO>;
   cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)fft_smem_bytes(pl.N));
   if (e != cudaSuccess) return e;
@@ -1048,11 +1037,16 @@ cudaError_t launch_fft_axis(double2* data, const FftPlan& pl, cudaStream_t st) {
   kern<<<grid, threads, fft_smem_bytes(pl.N), st>>>(data, pl);
   return cudaGetLastError();
 }
+cudaError_t launch_fft_axis(double2* data, const FftPlan& pl, cudaStream_t st) {
+  return launch_lines<FFT_FP64>(data, pl, st);
+}
 
 // Binned spectrum of a real field through the half spectrum: x-axis transform of
 // row pairs, y and z transforms of the N/2 + 1 columns kept, shell sums with the
 // conjugate partners counted, then eq. discretePS per bin (as launch_bins).
-// H holds (N/2 + 1) N^2 complex values; pl is the forward plan of N (tw set).
+// H holds (N/2 + 1) N^2 complex values, in fixed point until the last axis, and behind them
+// the exponents, N^2/2 of row pairs and (N/2 + 1) N of y-lines, and the powers (for N >= 8 all
+// within 2 N^3 complex values); pl is the forward plan of N (tw set).
 // The shell geometry of (N, dk) into bin_of (3 (N/2)^2 + 1 ints) and geo (2 nb
 // doubles: the sum of |n| and the count per bin); part holds 2 nb nblk doubles.
 cudaError_t launch_shell_geometry(int N, double dk, int nb, int nblk, int* bin_of, double* geo, double* part,
@@ -1068,16 +1062,21 @@ cudaError_t launch_shell_geometry(int N, double dk, int nb, int nblk, int* bin_o
   return cudaGetLastError();
 }
 
-cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftPlan& pl, double dk, int nb,
+cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftPlan& pl, int nb,
                                  int nblk, double* part, double kIR, double dx, double* out, cudaStream_t st,
                                  const int* bin_of, const double* geo) {
   const int N = pl.N;
   cudaError_t e;
+  int* const row_e = reinterpret_cast<int*>(H + (long long)(N / 2 + 1) * N * N);
+  int* const line_e = row_e + (long long)N * N / 2;
+  double* const power = reinterpret_cast<double*>(line_e + (long long)(N / 2 + 1) * N);  // an even number of ints
+  FftPlan pr = pl;
+  pr.eout = row_e;
   auto rows = [&](auto kern, auto* src) -> cudaError_t {
     const cudaError_t r = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)fft_smem_bytes(N));
     if (r != cudaSuccess) return r;
-    kern<<<(unsigned)((long long)N * N / 2 / pl.batch), fft_threads(N), fft_smem_bytes(N), st>>>(src, H, pl);
+    kern<<<(unsigned)((long long)N * N / 2 / pl.batch), fft_threads(N), fft_smem_bytes(N), st>>>(src, reinterpret_cast<CFix*>(H), pr);
     return cudaGetLastError();
   };
   if (fp32) {
@@ -1091,24 +1090,21 @@ cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftP
   }
   if (e != cudaSuccess) return e;
   FftPlan ph = fft_plan(N, pl.sign, pl.tw, N / 2 + 1, N / 2 + 1);
-  for (int axis = 1; axis < 3; ++axis) {
-    ph.axis = axis;
-    e = launch_fft_axis(H, ph, st);
-    if (e != cudaSuccess) return e;
-  }
-  if (bin_of && geo) {  // the cached shell geometry: only the power is summed
-    const int nc = std::max(1, std::min(16, (int)(48 * 1024 / (nb * sizeof(double)))));
-    bin_power_half_kernel<<<nblk, 512, nc * nb * sizeof(double), st>>>(H, bin_of, N, nb, nc, part);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    bin_final_geo_kernel<<<(nb + 3) / 4, 128, 0, st>>>(part, nblk, nb, geo, kIR, dx, N, out, out + nb,
-                                                            out + 2 * nb);
-    return cudaGetLastError();
-  }
-  bin_half_kernel<<<nblk, 256, 3 * nb * sizeof(double), st>>>(H, N, dk, nb, part);
+  ph.axis = 1;
+  ph.ein = row_e;
+  ph.eout = line_e;
+  e = launch_lines<FFT_FIX_FIX>(H, ph, st);
+  if (e != cudaSuccess) return e;
+  ph.axis = 2;
+  ph.ein = line_e;
+  ph.pout = power;
+  e = launch_lines<FFT_FIX_POWER>(H, ph, st);
+  if (e != cudaSuccess) return e;
+  const int nc = std::max(1, std::min(16, (int)(48 * 1024 / (nb * sizeof(double)))));
+  bin_power_half_kernel<<<nblk, 512, nc * nb * sizeof(double), st>>>(power, bin_of, N, nb, nc, part);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  bin_final_kernel<<<(nb + 127) / 128, 128, 0, st>>>(part, nblk, nb, kIR, dx, N, out, out + nb, out + 2 * nb, 0);
+  bin_final_geo_kernel<<<(nb + 3) / 4, 128, 0, st>>>(part, nblk, nb, geo, kIR, dx, N, out, out + nb, out + 2 * nb);
   return cudaGetLastError();
 }
 
