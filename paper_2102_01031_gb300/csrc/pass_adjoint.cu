@@ -34,8 +34,13 @@
 //
 // Same plane ring as the forward passes (ring.cuh): the stage holds
 // phi'_f, pi'_f (arrays 2f, 2f+1) and lam_phi'_f, lam_pi'_f (2NF + 2f, 2NF + 2f + 1).
+// FP64 storage is bound by its FP64 operations (64 cycles a warp each): both Laplacians in
+// integers (fix_lap.h), products of the potential shared, increments as FMAs: about 55 a
+// site of two fields for 95; gradient of 20 VV4 steps at 128^3 32600 -> 26400 us, at 96^3
+// 15750 -> 11800.
 #include "common.cuh"
 #include "ring.cuh"
+#include "fix_lap.h"
 #include "tail.cuh"
 
 namespace clg {
@@ -62,11 +67,20 @@ template <> struct AdjPot<2> {
   template <typename T>
   __device__ __forceinline__ static void eval(const T (&f)[2], T q, T (&d)[2], T (&H)[2][2], T (&dq)[2]) {
     const T p2 = f[0] * f[0], c2 = f[1] * f[1], pc = f[0] * f[1];
-    d[0] = p2 * f[0] + q * f[0] * c2;
-    d[1] = q * p2 * f[1];
-    H[0][0] = T(3) * p2 + q * c2;
-    H[0][1] = H[1][0] = T(2) * q * pc;
-    H[1][1] = q * p2;
+    if constexpr (sizeof(T) == 8) {  // the fewest FP64 operations
+      const T s = fmaT(q, c2, p2);
+      H[1][1] = q * p2;
+      d[0] = s * f[0];
+      d[1] = H[1][1] * f[1];
+      H[0][0] = fmaT(T(2), p2, s);
+      H[0][1] = H[1][0] = (T(2) * q) * pc;
+    } else {
+      d[0] = p2 * f[0] + q * f[0] * c2;
+      d[1] = q * p2 * f[1];
+      H[0][0] = T(3) * p2 + q * c2;
+      H[0][1] = H[1][0] = T(2) * q * pc;
+      H[1][1] = q * p2;
+    }
     dq[0] = f[0] * c2;
     dq[1] = p2 * f[1];
   }
@@ -150,6 +164,7 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const __grid_const
   constexpr int VX = V16<T>::n;
   constexpr int NA = 4 * NF;
   constexpr int LF = 2 * NF;  // first adjoint array
+  constexpr bool FP64 = sizeof(T) == 8;
   constexpr int NACC = SELF ? 4 : 1;
 
   extern __shared__ __align__(128) unsigned char smem[];
@@ -229,6 +244,7 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const __grid_const
           centre(sa, aF, aL);
           // Laplacians of phi' and l'
           T lapF[NF][VX], lapL[NF][VX];
+          bool in_range = true;  // FP64: the integer form holds
 #pragma unroll
           for (int k = 0; k < NF; ++k) {
 #pragma unroll
@@ -263,8 +279,38 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const __grid_const
                 const T cv = c[v];
                 const T xm = v == 0 ? left : c[v - 1];
                 const T xp = v == VX - 1 ? right : c[v + 1];
-                out[v] = ((xm + xp) - T(2) * cv) + ((yl[v] + yh[v]) - T(2) * cv) + ((b[v] + a[v]) - T(2) * cv);
+                if constexpr (FP64) {
+                  bool ok;
+                  out[v] = fix_lap(fix_val(xm), fix_val(xp), fix_val(yl[v]), fix_val(yh[v]), fix_val(b[v]), fix_val(a[v]),
+                                   fix_val(cv), &ok);
+                  in_range = in_range && ok;
+                } else {
+                  out[v] = ((xm + xp) - T(2) * cv) + ((yl[v] + yh[v]) - T(2) * cv) + ((b[v] + a[v]) - T(2) * cv);
+                }
               }
+            }
+          }
+          if constexpr (FP64) {
+            // the thread's sites again, in FP64 (one block of all of them: a branch, where a
+            // short one would be issued predicated and take its time on the FP64 unit)
+            if (!in_range) {
+#pragma unroll
+              for (int k = 0; k < NF; ++k)
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                  const T* base = sc + (m == 0 ? 2 * k : LF + 2 * k + 1) * ae;
+                  const T* pb = sc + (2 * k + 1) * ae;
+                  const T w = SELF && m == 1 ? bpost : T(0);
+                  auto at = [&](int e) { return m == 1 && SELF ? fmaT(w, pb[e], base[e]) : base[e]; };
+                  T (&c)[VX] = m == 0 ? cF[k] : cL[k];
+                  T (&b)[VX] = m == 0 ? bF[k] : bL[k];
+                  T (&a)[VX] = m == 0 ? aF[k] : aL[k];
+#pragma unroll
+                  for (int v = 0; v < VX; ++v)
+                    (m == 0 ? lapF : lapL)[k][v] =
+                        fp64_lap(v == 0 ? at((ty + 1) * N + xl) : c[v - 1], v == VX - 1 ? at((ty + 1) * N + xr) : c[v + 1],
+                                 at(ty * N + x0 + v), at((ty + 2) * N + x0 + v), b[v], a[v], c[v]);
+                }
             }
           }
           T npi[NF][VX], nphi[NF][VX], nlf[NF][VX], nlp[NF][VX];
@@ -283,10 +329,11 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const __grid_const
               T hl = T(0);
 #pragma unroll
               for (int m = 0; m < NF; ++m) hl = fmaT(H[k][m], cL[m][v], hl);
-              const T pi0 = pi1 - (A1 * lapF[k][v] - A3 * d[k]);
+              // FP32 adds the small increment last, FP64 takes two FMAs
+              const T pi0 = FP64 ? fmaT(-A1, lapF[k][v], fmaT(A3, d[k], pi1)) : pi1 - (A1 * lapF[k][v] - A3 * d[k]);
               npi[k][v] = pi0;
               nphi[k][v] = fmaT(-cd, pi0, f[k]);
-              T mu = lf1 + (A1 * lapL[k][v] - A3 * hl);
+              T mu = FP64 ? fmaT(A1, lapL[k][v], fmaT(-A3, hl, lf1)) : lf1 + (A1 * lapL[k][v] - A3 * hl);
               T lpre = cL[k][v];
               if (SELF) {
                 mu = fmaT(bphi, lapF[k][v], fmaT(bV, d[k], mu));
