@@ -44,12 +44,12 @@ PASSES_PER_STEP = 3
 # DRAM bytes (read + write) per DK pass from one ncu capture of the FP32 pass
 # at 256^3 (one cooperative launch of the three VV4 passes of a step, divided
 # by 3), valid only for the kernel source it was taken on.
-NCU_TRAFFIC = {"f32": {"source_hash": "e0b8777e15c09017", "bytes_per_launch": 503365461}}
+NCU_TRAFFIC = {"f32": {"source_hash": "1ed2df6a1b79dcdb", "bytes_per_launch": 505851477}}
 # FP64 instructions (DFMA, DADD, DMUL) and operations (FMA = 2) per site per pass
 # of the FP64 plain kernel, from one ncu capture of the instruction counters of
 # the FP64 pass at 256^3
-NCU_FP64_OPS = {"source_hash": "e0b8777e15c09017", "instructions_per_site_pass": 34.109,
-                "flops_per_site_pass": 49.144}
+NCU_FP64_OPS = {"source_hash": "1ed2df6a1b79dcdb", "instructions_per_site_pass": 17.126,
+                "flops_per_site_pass": 30.161}
 
 
 # Thread instructions per site of the doublet passes without expansion at the
@@ -58,13 +58,13 @@ NCU_FP64_OPS = {"source_hash": "e0b8777e15c09017", "instructions_per_site_pass":
 # leapfrog pass of 256^3 each) and their DRAM bytes per site (the same kernels
 # built for any N, one pass of 128^3), from ncu captures, valid for the kernel
 # source they were taken on.
-NCU_SU2 = {"source_hash": "85bf812048b7f8dc", "thread_instructions_per_site": 1400.0,
-           "dram_bytes_per_site": 268.8}
-NCU_FULL = {"source_hash": "85bf812048b7f8dc", "thread_instructions_per_site": 1616.3,
-            "dram_bytes_per_site": 318.0}
+NCU_SU2 = {"source_hash": "e76d458d3dd8f64e", "thread_instructions_per_site": 1377.5,
+           "dram_bytes_per_site": 268.2}
+NCU_FULL = {"source_hash": "e76d458d3dd8f64e", "thread_instructions_per_site": 1604.9,
+            "dram_bytes_per_site": 317.6}
 # The same for the U(1) pass without expansion at the benchmark size
 # (dk_pass_u1<float,0,true,256>, one leapfrog pass of 256^3).
-NCU_U1 = {"source_hash": "68ec87c02aca2e4a", "thread_instructions_per_site": 255.8,
+NCU_U1 = {"source_hash": "050f2db07dca54bd", "thread_instructions_per_site": 243.2,
           "dram_bytes_per_site": 80.4}
 # instruction issue of the whole GPU: 152 SMs x 4 schedulers x 32 lanes at the 2070 MHz maximum SM clock
 ISSUE_PEAK_LANE_INSTR_PER_S = 152 * 4 * 32 * 2.070e9
@@ -80,7 +80,7 @@ def u1_source_hash():
 
 def su2_source_hash():
     h = hashlib.sha256()
-    for name in ("pass_su2_kd.cu", "su2_common.cuh", "kd_drift.cuh", "trig2.cuh", "common.cuh", "tail.cuh"):
+    for name in ("pass_su2_kd.cu", "su2_kick.cuh", "su2_common.cuh", "kd_drift.cuh", "trig2.cuh", "common.cuh", "tail.cuh"):
         with open(os.path.join(ROOT, "paper_2102_01031_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -99,7 +99,7 @@ def kernel_source_hash():
     """Hash of the scalar pass kernel, its headers and the work split (what
     decides the pass's DRAM traffic and FP64 operation count)."""
     h = hashlib.sha256()
-    for name in ("pass_scalar.cu", "common.cuh", "tail.cuh", "worklist.h"):
+    for name in ("pass_scalar.cu", "ring.cuh", "fix_lap.h", "common.cuh", "tail.cuh", "worklist.h"):
         with open(os.path.join(ROOT, "paper_2102_01031_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -702,14 +702,14 @@ def other_workloads(P, torch, stream, peak):
         t_spec = (time.perf_counter() - t0) / reps
         lat.close()
         sites = N_LAT ** 3
-        gbs = sites * 52 / t_spec / 1e9
+        gbs = sites * 44 / t_spec / 1e9
         out["ics_and_spectrum_256_fp32"] = {
-            "init_s": t_init, "spectrum_ms": t_spec * 1e3, "model_bytes_per_site": 52,
+            "init_s": t_init, "spectrum_ms": t_spec * 1e3, "model_bytes_per_site": 44,
             "spectrum_gbs": gbs, "frac_hbm": gbs / peak,
-            "note": "host wall time; 52 B/site through the half spectrum = the FP32 field read 4 + the half "
-                    "spectrum written 8 by the x-axis transform + y and z axis passes 16 each + shell sums 8; "
-                    "includes the call's read-back and synchronisation; the transform is bound by its FP64 "
-                    "butterflies, not by memory"}
+            "note": "host wall time; 44 B/site through the half spectrum = the FP32 field read 4 + the half "
+                    "spectrum written 8 by the x-axis transform + y axis 16 + z axis read 8 and powers 4 + shell "
+                    "sums 4; includes the call's read-back and synchronisation; bound by the transforms' integer "
+                    "instructions, not by memory"}
     except Exception as e:  # noqa: BLE001
         out["ics_and_spectrum_256_fp32"] = {"error": str(e)[:300]}
     return out

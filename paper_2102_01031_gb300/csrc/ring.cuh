@@ -360,7 +360,7 @@ __device__ __forceinline__ bool ring_pass_begin(const Ring& R, const PassArgs& P
       else if (NUSED > 0) advance(base + lane);
     }
     if (NUSED > 0 && pass > 0) {
-      if (base > 0) __syncthreads();  // prep is this round's
+      if (base > 0) __syncthreads();  // prep holds these runs'
       if (warp == CONSUMER_WARPS - 2 && lane < nb && prep->fast) {
         const bool logs = blockIdx.x == 0;
         U::fast_powers(&rec[base + lane], prep, R.red + lane * NQ, logs ? pass_log(P, pass - 1, prep->lat) : nullptr,
