@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "fix_fft.h"   // FastDiv
+#include "friedmann.h"
 #include "worklist.h"  // Seg, MAX_SEG_PER_CTA
 
 #include "cl.h"
@@ -128,9 +129,10 @@ struct TailPrep {
   double wout, win, dnext;   // weights of the pass whose sums are taken
   double ckn, dnn;           // kick weight and drift of the pass that starts
   double pref, k[4];         // factors of the sums (the models' updates say which)
-  // fast (alpha = 1 with self-consistent expansion): b = a' after the two Friedmann kicks is
-  // b0 + c[0] s_kin + c[1] s_grad + c[2] s_pot of the pass's sums; a and pi2: the scale factor and sum of pi^2 before them
-  double b0, c[3], a, pi2;
+  // fast (alpha = 1 with self-consistent expansion): the two Friedmann kicks as a form of the
+  // pass's sums; a and pi2: the scale factor and sum of pi^2 before them
+  Alpha1Kick kick;
+  double a, pi2;
   int lat, fast;
 };
 // The bytes behind the stages for CTAs of at most nseg segments and nrun lattices,

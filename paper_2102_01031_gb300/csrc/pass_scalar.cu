@@ -146,13 +146,13 @@ struct ScalarUpdate {
   }
   // slot 1 holds sum phi Lap phi = -sum (grad^+ phi)^2
   __device__ __noinline__ static void fast_drift(Rec* r, const TailPrep* q, const double* sum) {
-    alpha1_drift(r->W, q, alpha1_b(q, sum[0], -sum[1], sum[2]));
+    alpha1_drift(r->W, q, alpha1_b(q->kick, sum[0], -sum[1], sum[2]));
     r->cf[0] = (T)r->W.cd;
     r->W.pi2 = sum[0];
   }
   __device__ __noinline__ static void fast_powers(Rec* r, const TailPrep* q, const double* sum, double* lgd,
                                                   double* lg) {
-    alpha1_powers(r->W, q, alpha1_b(q, sum[0], -sum[1], sum[2]));
+    alpha1_powers(r->W, q, alpha1_b(q->kick, sum[0], -sum[1], sum[2]));
     const double A1 = (q->ckn * r->L.inv_dx2) * r->W.apow1, A3 = q->ckn * r->W.apow3;
     r->cf[1] = (T)A1;
     r->cf[2] = (T)A3;
@@ -167,7 +167,7 @@ struct ScalarUpdate {
     }
     if (!lg) return;
     // the drift coefficient that fast_drift writes at the same time, formed alike
-    const double abar = fma(0.5 * q->dnext, alpha1_b(q, sum[0], -sum[1], sum[2]), q->a);
+    const double abar = fma(0.5 * q->dnext, alpha1_b(q->kick, sum[0], -sum[1], sum[2]), q->a);
     lg[0] = q->dnext == 0.0 ? 0.0 : q->dnext / (abar * abar);
     lg[1] = q->ckn;
     lg[2] = A1;

@@ -165,13 +165,13 @@ struct U1Update {
     if (L.expansion == CL_EXP_SELF) q->pref = kernel_a_pref(L, a);
   }
   __device__ __noinline__ static void fast_drift(Rec* r, const TailPrep* q, const double* sum) {
-    alpha1_drift(r->W, q, alpha1_b(q, sum[0], sum[1], sum[2]));
+    alpha1_drift(r->W, q, alpha1_b(q->kick, sum[0], sum[1], sum[2]));
     r->cf[0] = (T)r->W.cd;
     r->cf[1] = (T)r->W.cdA;
     r->W.pi2 = sum[0];  // pi2A, which enters with alpha - 1 = 0, stays
   }
   __device__ __noinline__ static void fast_powers(Rec* r, const TailPrep* q, const double* sum, double*, double*) {
-    alpha1_powers(r->W, q, alpha1_b(q, sum[0], sum[1], sum[2]));
+    alpha1_powers(r->W, q, alpha1_b(q->kick, sum[0], sum[1], sum[2]));
     const double k1 = q->ckn * r->W.apow1;
     r->cf[2] = (T)(k1 * r->L.inv_dx2);
     r->cf[3] = (T)(q->ckn * r->W.apow3);

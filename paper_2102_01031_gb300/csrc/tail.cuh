@@ -208,24 +208,14 @@ __device__ inline void advance_drift(double dn, const LatPar& L, SS& S) {
 // The same for alpha = 1 with self-consistent expansion.  Between two passes every
 // CTA waits for this, and on this part an FP64 operation takes about 100 cycles (64
 // even when it depends on nothing), so the work is cut to its dependent minimum:
-//   alpha1_ready, before the wait for the sums: with K_a = (a^3/3)(f_s/m_p)^2 [-E_K + E_G + 2 E_V],
-//     E_K = s_kin/(2 a^6 V), E_G = s_grad/(2 a^2 dx^2 V), E_V = s_pot/V, the kicked b as a
-//     linear form of the pass's sums (kin_pre: the pre-kick sum of pi^2);
+//   alpha1_ready, before the wait for the sums: the coefficients of the kicks of b (friedmann.h);
 //   then on two warps at once alpha1_drift (the division) and alpha1_powers.
 // One thread doing all of it took 4400 cycles between the sums and the next pass.
 __device__ __forceinline__ void alpha1_ready(const LatPar& L, const ScalarState& W, TailPrep* q) {
-  const double K = L.fm2 * (1.0 / 6.0) * L.inv_V, ws = q->wout + q->win;
-  const double a = W.a, a3 = a * a * a, k3 = K / a3;
   q->fast = 1;
-  q->a = a;
+  q->a = W.a;
   q->pi2 = W.pi2;
-  q->b0 = fma(-q->wout * k3, W.pi2, W.b);
-  q->c[0] = -q->win * k3;
-  q->c[1] = ws * (K * L.inv_dx2) * a;
-  q->c[2] = 4.0 * ws * K * a3;
-}
-__device__ __forceinline__ double alpha1_b(const TailPrep* q, double kin, double grad, double pot) {
-  return fma(q->c[0], kin, fma(q->c[1], grad, fma(q->c[2], pot, q->b0)));
+  q->kick = alpha1_kick(L.fm2 * (1.0 / 6.0) * L.inv_V, L.inv_dx2, W.a, W.b, W.pi2, q->wout, q->win);
 }
 // b and the drift coefficients at the midpoint scale factor
 __device__ __forceinline__ void alpha1_drift(ScalarState& W, const TailPrep* q, double b) {

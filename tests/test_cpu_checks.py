@@ -1,0 +1,22 @@
+"""CPU checks of arithmetic and host code that the kernels share with it (csrc headers), each
+a small program compiled with g++ that prints "OK" or what failed."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.mark.parametrize("name", ["friedmann_check"])
+def test_check_program(tmp_path, name):
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no g++")
+    exe = tmp_path / name
+    subprocess.run([gxx, "-O2", "-std=c++17", "-Wall", "-I", os.path.join(ROOT, "paper_2102_01031_gb300", "csrc"),
+                    os.path.join(ROOT, "tests", name + ".cpp"), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert r.stdout.splitlines()[-1].startswith("OK"), r.stdout
