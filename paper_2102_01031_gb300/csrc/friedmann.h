@@ -34,4 +34,7 @@ FX double alpha1_b(const Alpha1Kick& k, double kin, double grad, double pot) {
   return k.b + fma(k.c[0], kin, fma(k.c[1], grad, fma(k.c[2], pot, k.pre)));
 }
 
+// a after the drift by dn; a pass that closes a stream (dn = 0) leaves a as it is, whatever a' is.
+FX double alpha1_a(double dn, double b, double a) { return dn == 0.0 ? a : fma(dn, b, a); }
+
 }  // namespace clg

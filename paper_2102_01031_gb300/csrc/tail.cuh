@@ -227,7 +227,7 @@ __device__ __forceinline__ void alpha1_drift(ScalarState& W, const TailPrep* q, 
 }
 // a and its powers after the drift
 __device__ __forceinline__ void alpha1_powers(ScalarState& W, const TailPrep* q, double b) {
-  const double an = fma(q->dnext, b, q->a), an2 = an * an;
+  const double an = alpha1_a(q->dnext, b, q->a), an2 = an * an;
   W.a = an;
   if (q->dnext == 0.0) return;
   W.apow1 = an2;

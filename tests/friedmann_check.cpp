@@ -4,10 +4,12 @@
 // sizes (a coefficient takes at most 8 roundings: 3 for K, 3 for a^3 and the division or
 // 2 for a^3 and 1 for the weights' sum, and its products; the terms' sum 3, the last one
 // with the rounding of K's own factors to spare).
+// A pass without a drift leaves a as it is, also where a' is no number.
 // Then a homogeneous field's run: the error of a' stays that of the form that adds one
 // increment to it.  Prints "OK" or "FAIL ...".
 #include <cmath>
 #include <cstdio>
+#include <limits>
 #include <random>
 
 #include "friedmann.h"
@@ -42,6 +44,12 @@ int main() {
     if (!(off <= tol) && ++fails < 5)
       std::printf("FAIL case %d: off by %.3Lf units in the last place\n", n, off / std::ldexp(1.0L, e - 53));
   }
+  for (double b : {1.5, std::numeric_limits<double>::infinity(), std::nan("")})
+    if (alpha1_a(0.0, b, 2.5) != 2.5) {
+      ++fails;
+      std::printf("FAIL no drift, a' = %g: a = %g\n", b, alpha1_a(0.0, b, 2.5));
+    }
+  if (alpha1_a(0.01, 3.0, 2.5) != std::fma(0.01, 3.0, 2.5)) { ++fails; std::printf("FAIL drift\n"); }
   // phi^4/4 without gradients, leapfrog steps: a' against the same steps in extended precision,
   // and the form that adds the whole increment at once
   double sum_new = 0.0, sum_one = 0.0;
