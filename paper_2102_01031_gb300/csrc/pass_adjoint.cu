@@ -35,11 +35,11 @@
 // Same plane ring as the forward passes (ring.cuh): the stage holds
 // phi'_f, pi'_f (arrays 2f, 2f+1) and lam_phi'_f, lam_pi'_f (2NF + 2f, 2NF + 2f + 1).
 // FP64 storage is bound by its FP64 operations (64 cycles a warp each): both Laplacians in
-// integers (fix_lap.h), products of the potential shared, increments as FMAs: about 55 a
-// site of two fields for 95; gradient of 20 VV4 steps at 128^3 32600 -> 26400 us, at 96^3
-// 15750 -> 11800.
+// integers (fix_lap.h), products of the potential shared: about 60 a site of two fields for 95;
+// gradient of 20 VV4 steps at 128^3 32600 -> 26400 us, at 96^3 15750 -> 11800.
 #include "common.cuh"
 #include "ring.cuh"
+#include "adj_kick.h"
 #include "fix_lap.h"
 #include "tail.cuh"
 
@@ -329,11 +329,15 @@ __global__ void __launch_bounds__(THREADS, 1) adj_pass_scalar(const __grid_const
               T hl = T(0);
 #pragma unroll
               for (int m = 0; m < NF; ++m) hl = fmaT(H[k][m], cL[m][v], hl);
-              // FP32 adds the small increment last, FP64 takes two FMAs
-              const T pi0 = FP64 ? fmaT(-A1, lapF[k][v], fmaT(A3, d[k], pi1)) : pi1 - (A1 * lapF[k][v] - A3 * d[k]);
+              // the small increment last: one rounding at the momentum's size
+              T pi0;
+              if constexpr (FP64) pi0 = kicked(pi1, -A1, lapF[k][v], -A3, d[k]);
+              else pi0 = pi1 - (A1 * lapF[k][v] - A3 * d[k]);
               npi[k][v] = pi0;
               nphi[k][v] = fmaT(-cd, pi0, f[k]);
-              T mu = FP64 ? fmaT(A1, lapL[k][v], fmaT(-A3, hl, lf1)) : lf1 + (A1 * lapL[k][v] - A3 * hl);
+              T mu;
+              if constexpr (FP64) mu = kicked(lf1, A1, lapL[k][v], A3, hl);
+              else mu = lf1 + (A1 * lapL[k][v] - A3 * hl);
               T lpre = cL[k][v];
               if (SELF) {
                 mu = fmaT(bphi, lapF[k][v], fmaT(bV, d[k], mu));
