@@ -240,6 +240,22 @@ struct U1Update {
 
 }  // namespace
 
+// A pass's coefficients (U1Update::Rec::cf): LEAN reads them from shared memory where they are
+// used, else they are held in registers.
+template <typename T, bool LEAN> struct U1Coef {
+  T v[9];
+  __device__ __forceinline__ explicit U1Coef(const T* cf) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) v[k] = cf[k];
+  }
+  __device__ __forceinline__ T operator[](int k) const { return v[k]; }
+};
+template <typename T> struct U1Coef<T, true> {
+  const T* p;
+  __device__ __forceinline__ explicit U1Coef(const T* cf) : p(cf) {}
+  __device__ __forceinline__ T operator[](int k) const { return p[k]; }
+};
+
 // RED: 0 = no sums, 1 = sums for the Friedmann kick, 2 = full measurement, U1_RED_ALPHA1 =
 // the Friedmann kick's sums at alpha = 1, where the links' energies enter with alpha - 1 = 0
 // and are not formed (three half-angle sines a site and the momenta's squares).
@@ -265,6 +281,15 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
   constexpr int NACC = RED == 0 ? 1 : (RED == 1 ? 5 : (RED == U1_RED_ALPHA1 ? 3 : 12));
   constexpr int NUSED = RED == 0 ? 0 : (RED == 2 ? NQ : NACC);
   constexpr bool GS = RED == 1 || RED == 2;  // the links' sums
+  // FP32 passes with sums want more than the 128 registers a thread has.  They read their
+  // coefficients and the output pointer from shared memory where they use them and take the
+  // half-angle sines early, while the plaquette angles are at hand; the measurement without
+  // expansion takes them late and reads the x and y links of the plane above again when it
+  // becomes the current one.  With these values spilled in the marching loop a measurement at
+  // 256^3 took 468 us with self-consistent expansion (352 so) and 390 without (306), at 192^3
+  // 252 (189) and 231 (170), the step pass at alpha = 0 and 256^3 342 (312).  The other passes
+  // are as fast or faster with the values in registers (FP64 by 0.4 % at 128^3).
+  constexpr bool LEAN = sizeof(T) == 4 && RED > 0;
 
   extern __shared__ __align__(128) unsigned char smem[];
   const Ring R = ring_view(smem, P);
@@ -288,6 +313,11 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
   for (int pass = 0; pass < P.npass; ++pass) {
     const int parity = P.parity ^ (pass & 1);
     if (!ring_pass_begin<T, NAR, KD, NUSED, Update>(R, P, pass, ns, ptot, parity, false, warp, lane)) goto timeout;
+    if constexpr (RED == 2) {  // zeroed here too, the sums need no registers during the pass's begin
+#pragma unroll
+      for (int k = 0; k < NACC; ++k) acc[k].zero();
+      nonfinite = 0.f;
+    }
 
     for (int i = 0; i < ns; ++i) {
       const SegInfo& si = R.info[i];
@@ -302,17 +332,20 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
       const int mrow = KD ? -N : 0;  // KD: a momentum's stage rows start at the tile's first row
       const long long NN = (long long)N * N;
       const int g0 = R.off[i];
-      const T* const cf = rec[si.run].cf;
-      const T A1 = cf[2], A3 = cf[3], AJ = cf[4], AC = cf[5], gd = cf[6], v2 = cf[7], lam = cf[8];
+      const U1Coef<T, LEAN> cf(rec[si.run].cf);
       // KD: no deferred drift to apply on read, this pass's drift after its kick
-      const T cd = KD ? T(0) : cf[0], cdA = KD ? T(0) : cf[1], kd = KD ? cf[0] : T(0), kdA = KD ? cf[1] : T(0);
+      const T cd = KD ? T(0) : cf[0], cdA = KD ? T(0) : cf[1];
       const bool drifting = !KD && (cd != T(0) || cdA != T(0));
-      const V gdv = vset(gd);
       const int xl = x0 == 0 ? N - 1 : x0 - 1, xr = x0 + VX == N ? 0 : x0 + VX;
-      // output buffer: array a of a lattice buffer starts a * V elements after array 0
-      T* const dbase = static_cast<T*>(const_cast<void*>(si.src[parity ^ 1][0]));
-      const long long Vs = si.V;
-      const int z0 = si.z0, nz = si.nz;
+      // where the thread's sites of plane j go (segments march up and never wrap: plane j is
+      // z0 + j - 1); array a of a lattice buffer starts a * V elements after array 0
+      T* const held_base = static_cast<T*>(const_cast<void*>(si.src[parity ^ 1][0]));
+      const long long held_V = si.V;
+      const int held_z0 = si.z0;
+      auto out_of = [&](int j) -> T* {
+        T* const base = LEAN ? static_cast<T*>(const_cast<void*>(si.src[parity ^ 1][0])) : held_base;
+        return base + (long long)((LEAN ? si.z0 : held_z0) + j - 1) * NN + (long long)y * N + x0;
+      };
 
       // the thread's sites of field array a (its momentum is a + 1) on stage row `row`, drifted
       auto rdv = [&](const T* st, int a, int row, T coef) -> V {
@@ -347,7 +380,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
         azm = rdv(st, AZ, ty + 1, cdA);
         azm_yp = rdv(st, AZ, ty + 2, cdA);
         azm_xp = vxp(azm, right(st, AZ, ty + 1, cdA));
-        vsincos(vmul(gdv, azm), bSz, bCz);
+        vsincos(vmul(vset(cf[6]), azm), bSz, bCz);
       }
       ring_release<T, NAR, KD>(R, g0, s_cur, parity, ptot, lane);
       ring_advance(S, s_cur, p_cur);
@@ -359,6 +392,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
         cA0 = rdv(st, AX, ty + 1, cdA);
         cA1 = rdv(st, AY, ty + 1, cdA);
         cA2 = rdv(st, AZ, ty + 1, cdA);
+        const V gdv = vset(cf[6]);
         bSxz = vsin(plaq(gdv, axm, azm_xp, cA0, azm));
         bSyz = vsin(plaq(gdv, aym, azm_yp, cA1, azm));
       }
@@ -366,14 +400,25 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
       uint32_t p_nxt = p_cur;
       ring_advance(S, s_nxt, p_nxt);
 
-      for (int j = 1; j <= nz; ++j) {  // plane j in stage s_cur, plane j + 1 in s_nxt
+      for (int j = 1; j <= si.nz; ++j) {  // plane j in stage s_cur, plane j + 1 in s_nxt
         ring_wait(R, s_nxt, p_nxt, P.wait_limit_ns);
         if (active && !R.flag[0]) {
           const T* sa = ring_stage<T>(R, s_nxt);
           const T* sc = ring_stage<T>(R, s_cur);
           const int own = (ty + 1) * N + x0;
-          // segments march up and never wrap: plane j is z0 + j - 1
-          T* const out = dbase + (long long)(z0 + j - 1) * NN + (long long)y * N + x0;
+          T* const held_out = LEAN ? nullptr : out_of(j);
+          const T gd = cf[6];
+          const V gdv = vset(gd);
+          if constexpr (RED == 2) {
+#pragma unroll
+            for (int v = 0; v < VX; ++v) {
+              const T h0 = vget(cF0, v), h1 = vget(cF1, v);
+              acc[6].add(h0);
+              acc[7].add(h1);
+              acc[8].add(h0 * h0);
+              acc[9].add(h1 * h1);
+            }
+          }
           const V aF0 = rdv(sa, F0, ty + 1, cd), aF1 = rdv(sa, F1, ty + 1, cd);  // plane above, drifted
           const V aA0 = rdv(sa, AX, ty + 1, cdA), aA1 = rdv(sa, AY, ty + 1, cdA);
           const V ay_ym = rdv(sc, AY, ty, cdA), ay_ymzp = rdv(sa, AY, ty, cdA);
@@ -418,9 +463,22 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
           const V sym = sc4[3], cym = cc4[3];
           const V pxy = sn[0], pxz = sn[1], pyz = sn[2], sxy_ym = sn[3], syz_ym = sn[4];
           const V sxy_xm = vxm(pxy, vget(sn[5], 0)), sxz_xm = vxm(pxz, vget(sn[4 + NE], VX - 1));
+          auto magnetic = [&]() {  // 1 - cos of the plaquette angles
+            const V hxy = vsin(vmul(vset(T(0.5)), txy)), hxz = vsin(vmul(vset(T(0.5)), txz));
+            const V hyz = vsin(vmul(vset(T(0.5)), tyz));
+            T s_m = T(0);
+#pragma unroll
+            for (int v = 0; v < VX; ++v) {
+              const T hx = vget(hxy, v), hy = vget(hxz, v), hz = vget(hyz, v);
+              s_m += T(2) * (hx * hx + hy * hy + hz * hz);
+            }
+            if constexpr (GS) acc[RED == 1 ? 3 : 4].add(s_m);
+          };
+          if constexpr (GS && LEAN && !KD) magnetic();
           T s_g = T(0), s_v = T(0), s_pi = T(0);
           V Jx, Jy, Jz;
           // ---- charged scalar: covariant Laplacian, currents, potential, kick ----
+          const T A1 = cf[2], A3 = cf[3], v2 = cf[7], lam = cf[8];
           {
             const V fym0 = rdv(sc, F0, ty, cd), fym1 = rdv(sc, F1, ty, cd);
             const V fyp0 = rdv(sc, F0, ty + 2, cd), fyp1 = rdv(sc, F1, ty + 2, cd);
@@ -455,7 +513,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
               for (int v = 0; v < VX; ++v) {
                 const T e0 = vget(g0, v), e1 = vget(g1, v), e2 = vget(g2, v), e3 = vget(g3, v), e4 = vget(g4, v),
                         e5 = vget(g5, v);
-                const T q0 = vget(pn0, v), q1 = vget(pn1, v), h0 = vget(f0, v), h1 = vget(f1, v), d = vget(dd, v);
+                const T q0 = vget(pn0, v), q1 = vget(pn1, v), d = vget(dd, v);
                 s_g += e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3 + e4 * e4 + e5 * e5;
                 s_v += lam * d * d;
                 if constexpr (RED != 2) {
@@ -463,10 +521,6 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
                 } else {
                   acc[0].add(q0 * q0);
                   acc[1].add(q1 * q1);
-                  acc[6].add(h0);
-                  acc[7].add(h1);
-                  acc[8].add(h0 * h0);
-                  acc[9].add(h1 * h1);
                   acc[10].add(q0);
                   acc[11].add(q1);
                   if (!isfinite(q0) || !isfinite(q1)) nonfinite += 1.f;
@@ -474,9 +528,11 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
               }
             }
             if (P.write) {
+              T* const out = LEAN ? out_of(j) : held_out;
+              const long long Vs = LEAN ? si.V : held_V;
               if constexpr (KD) {
-                stv(out + F0 * Vs, vfma(vset(kd), pn0, f0));
-                stv(out + F1 * Vs, vfma(vset(kd), pn1, f1));
+                stv(out + F0 * Vs, vfma(vset(cf[0]), pn0, f0));
+                stv(out + F1 * Vs, vfma(vset(cf[0]), pn1, f1));
               } else {
                 stv(out + F0 * Vs, f0);
                 stv(out + F1 * Vs, f1);
@@ -486,7 +542,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
             }
           }
           // ---- links: currents, compact curl from plaquettes, kick ----
-          T s_piA = T(0), s_m = T(0);
+          T s_piA = T(0);
           {
             const V pax = *reinterpret_cast<const V*>(sc + aoff(PAX) + own + mrow);
             const V pay = *reinterpret_cast<const V*>(sc + aoff(PAY) + own + mrow);
@@ -494,28 +550,27 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
             const V Cx = vadd(vsub(pxy, sxy_ym), vsub(pxz, bSxz));
             const V Cy = vadd(vsub(sxy_xm, pxy), vsub(pyz, bSyz));
             const V Cz = vadd(vsub(sxz_xm, pxz), vsub(syz_ym, pyz));
-            const V AJv = vset(AJ), ACv = vset(AC);
+            const V AJv = vset(cf[4]), ACv = vset(cf[5]);
             const V pnx = vadd(pax, vfma(AJv, Jx, vmul(ACv, Cx)));
             const V pny = vadd(pay, vfma(AJv, Jy, vmul(ACv, Cy)));
             const V pnz = vadd(paz, vfma(AJv, Jz, vmul(ACv, Cz)));
             if constexpr (GS) {
-              const V hxy = vsin(vmul(vset(T(0.5)), txy)), hxz = vsin(vmul(vset(T(0.5)), txz));
-              const V hyz = vsin(vmul(vset(T(0.5)), tyz));
+              if constexpr (!LEAN || KD) magnetic();
 #pragma unroll
               for (int v = 0; v < VX; ++v) {
-                const T hx = vget(hxy, v), hy = vget(hxz, v), hz = vget(hyz, v);
                 const T qx = vget(pnx, v), qy = vget(pny, v), qz = vget(pnz, v);
-                s_m += T(2) * (hx * hx + hy * hy + hz * hz);
                 s_piA += qx * qx + qy * qy + qz * qz;
                 if constexpr (RED == 2)
                   if (!isfinite(qx) || !isfinite(qy) || !isfinite(qz)) nonfinite += 1.f;
               }
             }
             if (P.write) {
+              T* const out = LEAN ? out_of(j) : held_out;
+              const long long Vs = LEAN ? si.V : held_V;
               if constexpr (KD) {
-                stv(out + AX * Vs, vfma(vset(kdA), pnx, cA0));
-                stv(out + AY * Vs, vfma(vset(kdA), pny, cA1));
-                stv(out + AZ * Vs, vfma(vset(kdA), pnz, cA2));
+                stv(out + AX * Vs, vfma(vset(cf[1]), pnx, cA0));
+                stv(out + AY * Vs, vfma(vset(cf[1]), pny, cA1));
+                stv(out + AZ * Vs, vfma(vset(cf[1]), pnz, cA2));
               } else {
                 stv(out + AX * Vs, cA0);
                 stv(out + AY * Vs, cA1);
@@ -534,20 +589,18 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
             acc[0].add(s_pi);
             acc[1].add(s_piA);
             acc[2].add(s_g);
-            acc[3].add(s_m);
             acc[4].add(s_v);
           } else if constexpr (RED == 2) {
             acc[2].add(s_piA);
             acc[3].add(s_g);
-            acc[4].add(s_m);
             acc[5].add(s_v);
           }
           bF0 = cF0;
           bF1 = cF1;
           cF0 = aF0;
           cF1 = aF1;
-          cA0 = aA0;
-          cA1 = aA1;
+          cA0 = GS && LEAN && KD ? rdv(sa, AX, ty + 1, cdA) : aA0;
+          cA1 = GS && LEAN && KD ? rdv(sa, AY, ty + 1, cdA) : aA1;
           cA2 = rdv(sa, AZ, ty + 1, cdA);
           bCz = cz;
           bSz = sz;
@@ -559,7 +612,7 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
         p_cur = p_nxt;
         ring_advance(S, s_nxt, p_nxt);
       }
-      ring_release<T, NAR, KD>(R, g0 + nz + 1, s_cur, parity, ptot, lane);
+      ring_release<T, NAR, KD>(R, g0 + si.nz + 1, s_cur, parity, ptot, lane);
       ring_advance(S, s_cur, p_cur);
 
       if (!si.flush) continue;
