@@ -392,12 +392,17 @@ __device__ __forceinline__ void ring_pass_end(const Ring& R, const PassArgs& P, 
   for (int base = 0; base < npend; base += 32) {
     const int nb = min(32, npend - base);
     __threadfence();
+    // what the update needs besides the sums, by a warp that has none of the first sums to form
+    // (one lane after the sums instead took a single pass 1 to 2 us longer)
+    if (warp == 0 && lane < nb) {
+      const int r = R.pend[base + lane];
+      prep->lat = ring_run(R, ns, r).lat;
+      U::ready(P, pass, -1, &rec[r], prep);
+    }
     ring_slot_sums<NUSED>(R, P, pass, ns, nb, warp, lane, [&](int l) { return R.pend[base + l]; });
     __syncthreads();
     if (warp == CONSUMER_WARPS - 1 && lane < nb) {
-      const int r = R.pend[base + lane], lat = ring_run(R, ns, r).lat;
-      prep->lat = lat;
-      U::ready(P, pass, -1, &rec[r], prep);
+      const int r = R.pend[base + lane], lat = prep->lat;
       if (prep->fast) {
         U::fast_drift(&rec[r], prep, R.red + lane * NQ);
         U::fast_powers(&rec[r], prep, R.red + lane * NQ, pass_log(P, pass, lat), nullptr);
