@@ -17,6 +17,7 @@
 //   dJ/du(x) = 2 C_b Re[ sum_{n in b} F(n) e^{+ik.x} ].
 #include <algorithm>
 
+#include "adj_kick.h"
 #include "common.cuh"
 
 namespace clg {
@@ -32,7 +33,6 @@ __global__ void seed_chi_fraction_kernel(const LatConst* Lc, const LatScalars* S
   const double rho = S.obs.rho, J = (S.obs.EK[1] + S.obs.EG[1]) / rho;
   const double a = S.a, a2 = a * a, a6 = a2 * a2 * a2;
   const double kK = 1.0 / (a6 * (double)V * rho), kG = -L.inv_dx2 / (a2 * (double)V), q = L.q;
-  // divisions once, not per site (about ten FP64 operations each)
   const double iV = 1.0 / (double)V, irho = 1.0 / rho;
   const T* ph[2] = {reinterpret_cast<const T*>(L.buf[parity][0]), reinterpret_cast<const T*>(L.buf[parity][2])};
   const T* pm[2] = {reinterpret_cast<const T*>(L.buf[parity][1]), reinterpret_cast<const T*>(L.buf[parity][3])};
@@ -55,7 +55,7 @@ __global__ void seed_chi_fraction_kernel(const LatConst* Lc, const LatScalars* S
       const double dEG = kG * lap;
       const double chi = g == 1 ? 1.0 : 0.0;
       lp[g][n] = (T)((chi - J) * (double)pm[g][n] * kK);
-      lf[g][n] = (T)((chi * dEG - J * (dEG + d[g] * iV)) * irho);
+      lf[g][n] = (T)fraction_gradient<sizeof(T) == 8>(chi, J, dEG, d[g], (double)V, rho, iV, irho);
     }
     s += 0.5 * f0 * f0 * f1 * f1;
   }
