@@ -1011,9 +1011,21 @@ FftPlan fft_plan(int N, int sign, const int4* tw, int pitch, int nu) {
   return pl;
 }
 
-size_t fft_smem_bytes(int N) {
+constexpr size_t fft_smem_bytes(int N) {
   const size_t B = (size_t)fft_batch_of(N);
   return (2 * B * (N + 1) + N) * sizeof(CFix) + (B * (2 * sizeof(int) + sizeof(LineScale)) + 15) / 16 * 16;
+}
+// Lets a transform kernel take the shared memory of any lattice size: the limit is the
+// function's, and contexts of other sizes launch it from other host threads.
+constexpr size_t fft_smem_most() {
+  size_t m = 0;
+  for (int N = 8; N <= 512; N += 8)
+    if (fft_smem_bytes(N) > m) m = fft_smem_bytes(N);
+  return m;
+}
+static cudaError_t allow_fft_smem(const void* kern) {
+  static constexpr int most = (int)fft_smem_most();
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 // Threads per CTA: batch N <= 2048 elements, at most FFT_HELD a thread.
 int fft_threads(int N) { return std::max(64, (fft_batch_of(N) * N / FFT_HELD + 31) / 32 * 32); }
@@ -1029,8 +1041,7 @@ static cudaError_t launch_lines(double2* data, const FftPlan& pl, cudaStream_t s
                                           : pl.N == 256 ? fft_lines_kernel<256, IO>
                                           : pl.N == 512 ? fft_lines_kernel<512, IO>
                                                         : fft_lines_kernel<0, IO>;
-  cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fft_smem_bytes(pl.N));
+  cudaError_t e = allow_fft_smem((const void*)kern);
   if (e != cudaSuccess) return e;
   const int threads = fft_threads(pl.N);
   const unsigned grid = (unsigned)pl.ng * (unsigned)pl.N;
@@ -1073,8 +1084,7 @@ cudaError_t launch_real_spectrum(int fp32, const void* f, double2* H, const FftP
   FftPlan pr = pl;
   pr.eout = row_e;
   auto rows = [&](auto kern, auto* src) -> cudaError_t {
-    const cudaError_t r = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)fft_smem_bytes(N));
+    const cudaError_t r = allow_fft_smem((const void*)kern);
     if (r != cudaSuccess) return r;
     kern<<<(unsigned)((long long)N * N / 2 / pl.batch), fft_threads(N), fft_smem_bytes(N), st>>>(src, reinterpret_cast<CFix*>(H), pr);
     return cudaGetLastError();
