@@ -326,6 +326,8 @@ __device__ __forceinline__ void stockham_stage(const CFix* a, CFix* b, const int
 // The same with the line length N, the batch B and the sub-length Ns compiled in: for the
 // sizes runs are made at (128, 256, 512), where the index arithmetic of runtime sizes was a
 // fifth of the instructions (256^3: 223 -> 185 us for the row pairs, 194 -> 166 us an axis).
+// Other sizes and the rows of FP64 fields take the runtime-size kernels: a fifth of the rows' share
+// (20 of the 650 us of a 256^3 spectrum) for as many kernels again.
 template <int N, int B, int R, int Ns>
 __device__ __forceinline__ void stockham_stage_of(const CFix* a, CFix* b, const int4* w, int sign) {
   constexpr int NR = N / R, ts = N / (Ns * R), Pt = N + 1;
