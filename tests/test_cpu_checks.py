@@ -9,7 +9,7 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.mark.parametrize("name", ["friedmann_check", "adj_kick_check"])
+@pytest.mark.parametrize("name", ["friedmann_check", "adj_kick_check", "aligned_split_check"])
 def test_check_program(tmp_path, name):
     gxx = shutil.which("g++")
     if gxx is None:
