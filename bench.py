@@ -21,6 +21,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import signal
 import statistics
 import subprocess
@@ -70,20 +71,31 @@ NCU_U1 = {"source_hash": "050f2db07dca54bd", "thread_instructions_per_site": 243
 ISSUE_PEAK_LANE_INSTR_PER_S = 152 * 4 * 32 * 2.070e9
 
 
-def u1_source_hash():
+def source_hash(kernel, *split):
+    """Hash of a pass kernel's file, of every header beside it that it includes, directly or
+    through another one, and of the headers that split its work over the CTAs."""
+    csrc = os.path.join(ROOT, "paper_2102_01031_gb300", "csrc")
+    todo, text = [kernel, *split], {}
+    while todo:
+        name = todo.pop()
+        path = os.path.join(csrc, name)
+        if name in text or not os.path.exists(path):  # cl.h, the library's interface, lies elsewhere
+            continue
+        with open(path, "rb") as f:
+            text[name] = f.read()
+        todo += [m.decode() for m in re.findall(rb'^#include "([^"]+)"', text[name], re.M)]
     h = hashlib.sha256()
-    for name in ("pass_u1.cu", "ring.cuh", "kd_drift.cuh", "trig2.cuh", "common.cuh", "tail.cuh"):
-        with open(os.path.join(ROOT, "paper_2102_01031_gb300", "csrc", name), "rb") as f:
-            h.update(f.read())
+    for name in sorted(text):
+        h.update(name.encode() + b"\0" + text[name])
     return h.hexdigest()[:16]
+
+
+def u1_source_hash():
+    return source_hash("pass_u1.cu", "worklist.h")
 
 
 def su2_source_hash():
-    h = hashlib.sha256()
-    for name in ("pass_su2_kd.cu", "su2_kick.cuh", "su2_common.cuh", "kd_drift.cuh", "trig2.cuh", "common.cuh", "tail.cuh"):
-        with open(os.path.join(ROOT, "paper_2102_01031_gb300", "csrc", name), "rb") as f:
-            h.update(f.read())
-    return h.hexdigest()[:16]
+    return source_hash("pass_su2_kd.cu", "su2_work.h")
 
 
 def peaks():
@@ -96,13 +108,8 @@ def peaks():
 
 
 def kernel_source_hash():
-    """Hash of the scalar pass kernel, its headers and the work split (what
-    decides the pass's DRAM traffic and FP64 operation count)."""
-    h = hashlib.sha256()
-    for name in ("pass_scalar.cu", "ring.cuh", "fix_lap.h", "common.cuh", "tail.cuh", "worklist.h"):
-        with open(os.path.join(ROOT, "paper_2102_01031_gb300", "csrc", name), "rb") as f:
-            h.update(f.read())
-    return h.hexdigest()[:16]
+    """The scalar passes' (what decides their DRAM traffic and FP64 operation count)."""
+    return source_hash("pass_scalar.cu", "worklist.h")
 
 
 def ncu_fp64_ops():
