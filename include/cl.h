@@ -105,9 +105,14 @@ typedef struct {
   int precision;                /* CL_FP64 or CL_FP32 */
   void* stream;                 /* cudaStream_t */
   int autotune;                 /* nonzero: pick each lattice size's tile height by timing
-                                   candidates on the device (cached per model, precision, N) */
+                                   candidates on the device (cached per model, precision, N).
+                                   The timing runs enough lattices to fill the GPU; for one
+                                   small lattice the built-in choice, which may take a lower
+                                   tile to use more SMs, is the faster one */
   int tile_by;                  /* > 0: force this tile height (rows per CTA tile) for every
-                                   lattice; 0: autotune or the built-in choice */
+                                   lattice; 0: autotune or the built-in choice.  Lowered only
+                                   where a CTA works on so many lattices that its records leave
+                                   no room for three ring stages (see cl_lattice_tile) */
   double gQB;                   /* SU(2) coupling times charge (g_B Q_B), CL_MODEL_SU2U1_HIGGS */
   double qG, qH;                /* CL_MODEL_LPHI4_SU2U1: q_G = g^2/lambda, q_H = h^2/lambda (eq. PotGauge) */
   double Qc;                    /* CL_MODEL_LPHI4_SU2U1: U(1) charge of vphi in units of the doublet's

@@ -346,8 +346,10 @@ size_t stage_size(int N, int BY, int narr, int esz, bool mown = false) {
 // the own sites only, so their stages hold the momenta without halo rows.
 bool ring_mown(const cl_ctx* c) { return c->model == CL_MODEL_U1_HIGGS && c->p.expansion != CL_EXP_SELF; }
 
-// Shared memory that tile_candidates sets aside behind the stages: what a CTA of
-// MAX_SEG_PER_CTA segments over a few dozen lattices needs.
+// Shared memory that tile_candidates sets aside behind the stages.  It decides which heights
+// tile_by and tuned files may name, so it stays what it was when the bytes behind the stages did
+// not depend on the split.  A split's own (sm_tail_bytes) are 6.4 KB for a single lattice and
+// up to 53 KB for a CTA of 64 segments on as many lattices; init_impl sizes the ring by them.
 constexpr size_t SM_TAIL_RESERVE = 17408;
 
 // Tile heights BY admissible for N: BY divides N, the BY rows of N/VX
@@ -955,7 +957,8 @@ static cl_status init_impl(cl_ctx* c, const int* Ns, const double* kIRs, const u
   }
   // stage ring: the largest lattice stage, as many stages (3 .. 6) as fit beside the
   // CTAs' records; where a CTA's records of very many lattices leave fewer than three,
-  // the lattices of the largest stage take the next lower tile
+  // the lattices of the largest stage take the next lower tile (also a given or tuned one:
+  // cl_lattice_tile tells)
   size_t tail = 0;
   int S = 0;
   for (;;) {

@@ -15,13 +15,13 @@
 // array streams into a ring of shared-memory stages by 1-D bulk async copies
 // (TMA), completion counted on the stage's mbarrier.  The 16 warps never meet
 // at a block barrier while marching: each waits for the stage it needs,
-// applies the drift in registers as it reads (z-neighbours stay in registers,
-// y-neighbours come from the stage, x-neighbours from warp shuffles), kicks,
-// stores, and releases the stage; the last warp to release a stage (shared
-// memory count) issues the copies of the plane S places further in the
-// sequence, so the ring runs on across segment boundaries.  Sums are formed
-// per plane in the storage precision, added once per plane to compensated
-// (FP32) or plain (FP64) accumulators and flushed once per run into the run's
+// applies the drift in registers as it reads (z-neighbours and the thread's own
+// sites stay in registers, y-neighbours and the x-neighbours beyond its own sites
+// come from the stage), kicks, stores, and releases the stage; the last warp to
+// release a stage (shared memory count) issues the copies of the plane S places
+// further in the sequence, so the ring runs on across segment boundaries.  FP32
+// sums are formed per plane and added once per plane to compensated accumulators,
+// FP64 sums site by site to plain ones, and flushed once per run into the run's
 // slot; between two passes every CTA sums its lattices' slots in a fixed order
 // and runs their Friedmann update itself (ring.cuh, tail.cuh).
 //

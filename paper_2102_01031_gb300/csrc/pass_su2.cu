@@ -43,7 +43,7 @@
 // site, 41 % of the issue slots; memory alone takes 350 of 940 us at 192^3).  The kick is
 // the kick-then-drift passes' (su2_kick.cuh: each plaquette once, carried along z), one
 // barrier a plane, and at alpha = 1 no gauge energies: lphi4SU2U1 192^3 FP32, 5 VV2 steps
-// and energies 6399 -> 5870 us, the measurement pass alone 1323 -> 1161 us.
+// and energies 6399 -> 5900 us, the measurement pass alone 1323 -> 1161 us.
 #include "su2_kick.cuh"
 
 namespace clg {

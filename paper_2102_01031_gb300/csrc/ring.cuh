@@ -149,8 +149,10 @@ __device__ __forceinline__ const T* ring_stage(const Ring& R, int s) {
 // copied without their halo rows -- the tile's own rows only, one run -- and
 // each (field, momentum) pair occupies rows + (rows - 2) rows of the stage,
 // the field's first.
-// Stage memory is only read through the generic proxy and its reuse is
-// ordered by the release count, so no proxy fence precedes the copies.
+// The reuse of stage memory is ordered by the release count.  The passes read it through the
+// generic proxy, and a copy needs no proxy fence after reads; the FP64 scalar pass also writes
+// drifted values into it, and fences them itself before it releases the stage
+// (fence_proxy_async_smem in pass_scalar.cu).
 template <typename T, int NA, bool MOWN = false>
 __device__ void ring_issue_warp(const Ring& R, int g, int s, int parity, int lane) {
   static_assert(3 * NA <= 32, "one lane per copy");
