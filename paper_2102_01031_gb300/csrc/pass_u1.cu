@@ -287,9 +287,12 @@ __global__ void __launch_bounds__(THREADS, 1) dk_pass_u1(const __grid_constant__
   // expansion takes them late and reads the x and y links of the plane above again when it
   // becomes the current one.  With these values spilled in the marching loop a measurement at
   // 256^3 took 468 us with self-consistent expansion (352 so) and 390 without (306), at 192^3
-  // 252 (189) and 231 (170), the step pass at alpha = 0 and 256^3 342 (312).  The other passes
-  // are as fast or faster with the values in registers (FP64 by 0.4 % at 128^3).
-  constexpr bool LEAN = sizeof(T) == 4 && RED > 0;
+  // 252 (189) and 231 (170), the step pass at alpha = 0 and 256^3 342 (312).  FP64 passes with
+  // the links' sums gain by it where their spills miss L1 (measurement and step pass at
+  // alpha = 0: 288^3 23360 -> 23165 and 22880 -> 22330 us, 216^3 9645 -> 9625 and 9480 -> 9370)
+  // and lose 0.2 and 0.4 % at 128^3.  The other passes are as fast or faster with the values
+  // in registers (FP64 without the links' sums by 0.4 % at 128^3).
+  constexpr bool LEAN = sizeof(T) == 4 ? RED > 0 : GS;
 
   extern __shared__ __align__(128) unsigned char smem[];
   const Ring R = ring_view(smem, P);
