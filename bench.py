@@ -45,11 +45,11 @@ PASSES_PER_STEP = 3
 # DRAM bytes (read + write) per DK pass from one ncu capture of the FP32 pass
 # at 256^3 (one cooperative launch of the three VV4 passes of a step, divided
 # by 3), valid only for the kernel source it was taken on.
-NCU_TRAFFIC = {"f32": {"source_hash": "1ed2df6a1b79dcdb", "bytes_per_launch": 505851477}}
+NCU_TRAFFIC = {"f32": {"source_hash": "47da850086fe3dc3", "bytes_per_launch": 506343083}}
 # FP64 instructions (DFMA, DADD, DMUL) and operations (FMA = 2) per site per pass
 # of the FP64 plain kernel, from one ncu capture of the instruction counters of
 # the FP64 pass at 256^3
-NCU_FP64_OPS = {"source_hash": "1ed2df6a1b79dcdb", "instructions_per_site_pass": 17.126,
+NCU_FP64_OPS = {"source_hash": "47da850086fe3dc3", "instructions_per_site_pass": 17.126,
                 "flops_per_site_pass": 30.161}
 
 
@@ -59,14 +59,14 @@ NCU_FP64_OPS = {"source_hash": "1ed2df6a1b79dcdb", "instructions_per_site_pass":
 # leapfrog pass of 256^3 each) and their DRAM bytes per site (the same kernels
 # built for any N, one pass of 128^3), from ncu captures, valid for the kernel
 # source they were taken on.
-NCU_SU2 = {"source_hash": "e76d458d3dd8f64e", "thread_instructions_per_site": 1377.5,
-           "dram_bytes_per_site": 268.2}
-NCU_FULL = {"source_hash": "e76d458d3dd8f64e", "thread_instructions_per_site": 1604.9,
-            "dram_bytes_per_site": 317.6}
+NCU_SU2 = {"source_hash": "ac6eb3d17b3ab04b", "thread_instructions_per_site": 1384.5,
+           "dram_bytes_per_site": 268.3}
+NCU_FULL = {"source_hash": "ac6eb3d17b3ab04b", "thread_instructions_per_site": 1604.9,
+            "dram_bytes_per_site": 317.7}
 # The same for the U(1) pass without expansion at the benchmark size
 # (dk_pass_u1<float,0,true,256>, one leapfrog pass of 256^3).
-NCU_U1 = {"source_hash": "050f2db07dca54bd", "thread_instructions_per_site": 243.2,
-          "dram_bytes_per_site": 80.4}
+NCU_U1 = {"source_hash": "b48a0d43ba53e09e", "thread_instructions_per_site": 244.7,
+          "dram_bytes_per_site": 80.5}
 # instruction issue of the whole GPU: 152 SMs x 4 schedulers x 32 lanes at the 2070 MHz maximum SM clock
 ISSUE_PEAK_LANE_INSTR_PER_S = 152 * 4 * 32 * 2.070e9
 
@@ -735,9 +735,10 @@ def profile_case(name):
         lat = P.Lattice(P.MODEL_LPHI4_CHI, N_LAT, KIR, ALPHA, SEED,
                         P.make_params(precision=P.FP32, stream=stream, **PARAMS))
         lat.step(1)
-    elif name == "u1_128":    # single-pass launches of the leapfrog U(1) pass
-        u1 = dict(dt=0.01, integrator=P.LF, lam=1.0, v=1.0, gQ=0.5, fstar_over_omegastar=1.0,
-                  phi0=[1.0, 1.0], fluct_amp2=1e-2, expansion=P.EXP_OFF, fstar_over_mp=0.5)
+    elif name in ("u1_128", "u1_128self"):    # single-pass launches of the leapfrog U(1) pass
+        u1 = dict(dt=0.01, integrator=P.LF, lam=1.0, v=1.0 if name == "u1_128" else 0.0, gQ=0.5,
+                  fstar_over_omegastar=1.0, phi0=[1.0, 1.0], fluct_amp2=1e-2,
+                  expansion=P.EXP_OFF if name == "u1_128" else P.EXP_SELF, fstar_over_mp=0.5)
         lat = P.Lattice(P.MODEL_U1_HIGGS, 128, 0.2, ALPHA, SEED, P.make_params(precision=P.FP32, stream=stream, **u1))
         for _ in range(4):
             lat.step(1)
@@ -763,10 +764,11 @@ def profile_case(name):
                                                                                qH=0.8, Qc=0.7)))
         for _ in range(4):
             lat.step(1)
-    elif name == "full_128":  # single-pass launches of the leapfrog lphi4SU2U1 pass
+    elif name in ("full_128", "full_128self"):  # single-pass launches of the lphi4SU2U1 pass
+        exp = P.EXP_OFF if name == "full_128" else P.EXP_SELF
         lat = P.Lattice(P.MODEL_LPHI4_SU2U1, 128, 0.2, ALPHA, SEED,
                         P.make_params(precision=P.FP32, stream=stream,
-                                      **dict(su2_params(P), v=0.0, qG=1.5, qH=0.8, Qc=0.7)))
+                                      **dict(su2_params(P), v=0.0, qG=1.5, qH=0.8, Qc=0.7, expansion=exp)))
         for _ in range(4):
             lat.step(1)
     elif name == "ensemble64":   # the 64-lattice ensemble: one cooperative launch of a VV4 step
@@ -813,8 +815,9 @@ def main():
     ap.add_argument("--ref-budget", type=float, default=150.0,
                     help="reference arm: site-steps budget / 1e6 that sizes its oracle box")
     ap.add_argument("--no-extra", action="store_true", help="skip the U(1), ensemble and adjoint rows")
-    ap.add_argument("--profile-case", choices=("scalar256", "scalar256_fp64", "u1_128", "u1_256", "su2_128", "full_128", "su2_256", "full_256",
-                             "adj128", "adj128self", "spectrum256", "ensemble64"),
+    ap.add_argument("--profile-case", choices=("scalar256", "scalar256_fp64", "u1_128", "u1_128self", "u1_256", "su2_128",
+                                                    "full_128", "full_128self", "su2_256", "full_256", "adj128",
+                                                    "adj128self", "spectrum256", "ensemble64"),
                     help="run one small case for an ncu capture and exit")
     args = ap.parse_args()
     if args.profile_case:
