@@ -36,7 +36,7 @@
 // phi'_f, pi'_f (arrays 2f, 2f+1) and lam_phi'_f, lam_pi'_f (2NF + 2f, 2NF + 2f + 1).
 // FP64 storage is bound by its FP64 operations (64 cycles a warp each): both Laplacians in
 // integers (fix_lap.h), products of the potential shared: about 60 a site of two fields for 95;
-// gradient of 20 VV4 steps at 128^3 32600 -> 26400 us, at 96^3 15750 -> 11800.
+// gradient of 20 VV4 steps at 128^3 32600 -> 27700 us, at 96^3 15750 -> 12300.
 #include "common.cuh"
 #include "ring.cuh"
 #include "adj_kick.h"

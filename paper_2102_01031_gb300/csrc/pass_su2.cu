@@ -39,11 +39,11 @@
 // loads with the other's arithmetic.  The last CTA to finish sums the per-CTA
 // partial sums in a fixed order and advances the scale factor (tail.cuh).
 //
-// Bound by issue slots and the latency of a halo site's loads (about 2200 instructions a
-// site, 41 % of the issue slots; memory alone takes 350 of 940 us at 192^3).  The kick is
+// Bound by the latency of a halo site's loads and the plane's barrier behind them (2320
+// instructions a site, 44 % of the issue slots; memory alone takes 350 of 940 us at 192^3).  The kick is
 // the kick-then-drift passes' (su2_kick.cuh: each plaquette once, carried along z), one
 // barrier a plane, and at alpha = 1 no gauge energies: lphi4SU2U1 192^3 FP32, 5 VV2 steps
-// and energies 6399 -> 5900 us, the measurement pass alone 1323 -> 1161 us.
+// and energies 6457 -> 5992 us, the measurement pass alone 1323 -> 1161 us.
 #include "su2_kick.cuh"
 
 namespace clg {
